@@ -128,7 +128,9 @@ int lbm_workspace_bytes(const lbm_params* p, uint64_t* bytes);
 int lbm_init(const lbm_params* p, const double* rho0, int rho0_where, void* stream, lbm_handle** out);
 
 /* Advance nsteps >= 0 time steps (asynchronous on the handle's stream). Each step is
- * one launch of the fused kernel: stream (and, with Zou-He walls, rebuild the wall nodes'
+ * one launch of a fused kernel - with every relaxation time 1 and the default tile one that
+ * holds the state between calls as rho and j of the streamed populations, from which the
+ * populations are formed when they are read: stream (and, with Zou-He walls, rebuild the wall nodes'
  * incoming populations), rho, psi, <rho>, F_int, F_g, u, MRT + Li forcing, store. Device-side faults (non-physical state, timeouts) are recorded in a
  * sticky status returned by the next synchronising call.
  * Thermal variant: psi uses R T(x) of the current temperature field T^n, and the step
@@ -187,7 +189,8 @@ int lbm_coexistence(double a, double b, double R, double T, double* rho_v, doubl
 
 /* Launch configuration the handle uses for its fused step (for reports and tests):
  * grid CTAs, threads per CTA, dynamic shared bytes, band width (nodes along x per CTA),
- * strip height (rows per CTA), pipeline stages. Any pointer may be NULL. */
+ * strip height (rows per CTA), pipeline stages - of the step on populations. Any pointer may be
+ * NULL. */
 int lbm_launch_info(const lbm_handle* h, int* grid, int* block, int* smem_bytes,
                     int* band_width, int* strip_rows, int* stages);
 

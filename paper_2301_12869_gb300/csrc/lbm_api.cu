@@ -138,6 +138,16 @@ struct lbm_handle {
   void* Tnext = nullptr; // the field after the next energy step (swapped with Tf)
   bool have_prev = false;
   int64_t steps = 0;
+  // The step on moments (lbm_walk.cu). The state is held as the populations f[cur] (pop), as the
+  // moments m(mcur) of the next step's streamed populations (mom), or both. The moment buffers
+  // m(0), m(1) lie in f[1 - cur]; parts[b] holds the partial sums of m(b) while mom is set, and
+  // the populations f[cur] can be formed from m(1 - mcur), the state before the last step.
+  lbm::WalkTiling walk{};
+  bool pop = true, mom = false;
+  int mcur = 0;
+  int since_io = 0;      // population steps since the populations were last set or read
+  void* m(int b) const { return static_cast<char*>(f[1 - cur]) + size_t(3 * b) * N * s; }
+  double* mean(int b) const { return red + 4 + b; }  // Zou-He: <rho> - rho_ref for the collision of m(b)
   lbm::StepTiling tiling{};
   lbm::StepPhys phys{};
   double rho_mid = NAN;
@@ -308,11 +318,75 @@ int device_status(lbm_handle* h) {
   return LBM_OK;
 }
 
+// ---- the two forms of a handle's state
+// Fewest steps from a populations state for which the moments are formed: the change of form
+// costs a pull (48 B a node) and, when the populations are read, a collision (48 B) on top of
+// 24 B a step against the population step's 72 B, so it pays from two steps on; up to four,
+// its two launches cost a small lattice what the steps save.
+constexpr int kWalkSteps = 4;
+
+// The step on moments needs every relaxation time 1 and the default tile. FP64 lattices below
+// 2^16 nodes keep the population step: a walk's row takes 5 us of one warp's FP64 instructions
+// (4 x 200: 31.6 us a step against 13.6; 256 x 256: 48.6 against 52.1).
+bool walk_usable(const lbm_handle* h) {
+  return lbm::unit_relaxation(h->phys) && (h->p.precision == LBM_FP32 || h->N >= (size_t(1) << 16));
+}
+bool walk_eligible(const lbm_handle* h) { return h->tiling.variant == 0 && walk_usable(h); }
+
+lbm::WalkIO walk_io(lbm_handle* h, int b) {  // reading m(b)
+  lbm::WalkIO io{};
+  io.min = h->m(b);
+  io.part_in = h->parts[b];
+  io.npart_in = h->walk.ctas;
+  io.mean_in = h->mean(b);
+  io.status = h->status;
+  return io;
+}
+
+// m(0) = the moments of the populations f[cur]
+int form_moments(lbm_handle* h) {
+  if (h->mom) return LBM_OK;
+  lbm::WalkIO io{};
+  io.fin = h->f[h->cur];
+  io.mout = h->m(0);
+  io.part_in = h->parts[h->pcur];
+  io.npart_in = h->npart;
+  if (h->pcur == 0) std::swap(h->parts[0], h->parts[1]), h->pcur = 1;  // the sums read are not m(0)'s
+  io.part_out = h->parts[0];
+  io.mean_out = h->mean(0);
+  io.status = h->status;
+  LBM_CUDA(h, lbm::launch_pull(h->p.precision, h->walk, h->phys, io, h->stream));
+  h->mom = true;
+  h->mcur = 0;
+  return LBM_OK;
+}
+
+// the populations f[cur] of a state held as moments: the collision of the state before
+int form_populations(lbm_handle* h) {
+  h->since_io = 0;
+  if (h->pop) return LBM_OK;
+  lbm::WalkIO io = walk_io(h, 1 - h->mcur);
+  io.fout = h->f[h->cur];
+  io.Tfield = h->Tnext;  // the temperature that step used
+  LBM_CUDA(h, lbm::launch_walk(h->p.precision, lbm::WALK_POPULATIONS, h->walk, h->phys, io, h->stream));
+  h->pop = true;
+  return LBM_OK;
+}
+
 // Fresh FP64 partials of the stored state into parts[pcur].
 int refresh_partials(lbm_handle* h) {
   LBM_CUDA(h, lbm::launch_partials(h->p.precision, h->f[h->cur], h->p.nx, h->p.ny, h->parts[h->pcur], h->P, h->stream));
   h->npart = h->P;
   return LBM_OK;
+}
+
+// the state as populations alone, with their partial sums
+int leave_moments(lbm_handle* h) {
+  if (!h->mom) return LBM_OK;
+  int rc = form_populations(h);
+  if (rc) return rc;
+  h->mom = false;
+  return refresh_partials(h);
 }
 
 // A thermal step stores its rho, u for the energy equation in the handle's moment
@@ -330,7 +404,55 @@ void set_thermal_outputs(lbm_handle* h, lbm::StepIO& io) {
   }
 }
 
+int energy_step(lbm_handle* h) {
+  // T^n -> T^(n+1) with the rho^n, u^n this step formed (force of T^n)
+  const lbm_params& p = h->p;
+  LBM_CUDA(h, lbm::launch_energy_step(p.precision, p.nx, p.ny, p.wall == LBM_WALL_ZOU_HE ? 1 : 0, p.R, p.b, p.c_v,
+                                      p.kappa, p.T_bot, p.T_top, h->rho_now, h->ux, h->uy, h->Tf, h->Tnext, h->stream));
+  std::swap(h->Tf, h->Tnext);
+  return LBM_OK;
+}
+
+// one launch m(mcur) -> m(1 - mcur)
+int walk_launch(lbm_handle* h) {
+  lbm::WalkIO io = walk_io(h, h->mcur);
+  io.mout = h->m(1 - h->mcur);
+  io.part_out = h->parts[1 - h->mcur];
+  io.mean_out = h->mean(1 - h->mcur);
+  io.Tfield = h->Tf;
+  if (h->p.thermal) {
+    io.rho_T = h->rho_now;
+    io.ux_T = h->ux;
+    io.uy_T = h->uy;
+  }
+  LBM_CUDA(h, lbm::launch_walk(h->p.precision, lbm::WALK_STEP, h->walk, h->phys, io, h->stream));
+  h->mcur = 1 - h->mcur;
+  return LBM_OK;
+}
+
+int walk_steps(lbm_handle* h, int64_t nsteps) {
+  if (nsteps == 0) return LBM_OK;
+  if (int rc = form_moments(h)) return rc;
+  for (int64_t t = 0; t < nsteps; ++t) {
+    if (int rc = walk_launch(h)) return rc;
+    h->pop = false;
+    ++h->steps;
+    if (h->p.thermal)
+      if (int rc = energy_step(h)) return rc;
+  }
+  return LBM_OK;
+}
+
 int run_moments(lbm_handle* h, double* rho, double* ux, double* uy) {
+  if (h->mom) {
+    lbm::WalkIO io = walk_io(h, h->mcur);
+    io.Tfield = h->Tf;
+    io.rho_out = rho;
+    io.ux_out = ux;
+    io.uy_out = uy;
+    LBM_CUDA(h, lbm::launch_walk(h->p.precision, lbm::WALK_MOMENTS, h->walk, h->phys, io, h->stream));
+    return LBM_OK;
+  }
   lbm::StepIO io{};
   io.Tfield = h->Tf;
   io.fin = h->f[h->cur];
@@ -466,6 +588,7 @@ int lbm_init(const lbm_params* p, const double* rho0, int rho0_where, void* stre
   h->P = h->tiling.nbands * h->tiling.nstrips;
   h->Pcap = max_partials(*p, h->nsm, h->err);
   if (h->Pcap < 0) return fail(LBM_EINVAL);
+  lbm::plan_walk(p->precision, p->nx, p->ny, p->wall == LBM_WALL_ZOU_HE, h->nsm, h->Pcap, &h->walk);
   const Layout L = layout_for(*p, h->Pcap);
   if (p->workspace) {
     if (p->workspace_bytes < L.total || (reinterpret_cast<uintptr_t>(p->workspace) & 255)) {
@@ -545,6 +668,9 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
   lbm::TraceRange trace("lbm_step");
   if (!h) { set_err(g_err, "handle is NULL"); return LBM_EINVAL; }
   if (nsteps < 0) { set_err(h->err, "nsteps must be >= 0"); return LBM_EINVAL; }
+  if (walk_eligible(h) && (h->mom || nsteps + h->since_io >= kWalkSteps)) return walk_steps(h, nsteps);
+  if (int rc = leave_moments(h)) return rc;
+  h->since_io = int(std::min<int64_t>(h->since_io + nsteps, kWalkSteps));
   lbm::StepIO io{};
   io.status = h->status;
   const lbm_params& p = h->p;
@@ -561,13 +687,8 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
     h->pcur = 1 - h->pcur;
     h->npart = h->P;
     ++h->steps;
-    if (p.thermal) {
-      // T^n -> T^(n+1) with the rho^n, u^n this step formed (force of T^n)
-      LBM_CUDA(h, lbm::launch_energy_step(p.precision, p.nx, p.ny, p.wall == LBM_WALL_ZOU_HE ? 1 : 0, p.R, p.b, p.c_v,
-                                          p.kappa, p.T_bot, p.T_top, h->rho_now, h->ux, h->uy, h->Tf, h->Tnext,
-                                          h->stream));
-      std::swap(h->Tf, h->Tnext);
-    }
+    if (p.thermal)
+      if (int rc = energy_step(h)) return rc;
   }
   return LBM_OK;
 }
@@ -595,7 +716,9 @@ int lbm_reduce(lbm_handle* h, int kind, double* out) {
   switch (kind) {
     case LBM_REDUCE_MASS:
     case LBM_REDUCE_MEAN_RHO: {
-      double* scratch = h->parts[1 - h->pcur];  // overwritten by the next step anyway
+      if ((rc = form_populations(h))) return rc;
+      // overwritten by the next step anyway (ux: as many slots as nodes, at least one per CTA)
+      double* scratch = h->mom ? h->ux : h->parts[1 - h->pcur];
       LBM_CUDA(h, lbm::launch_partials(h->p.precision, h->f[h->cur], nx, ny, scratch, h->P, h->stream));
       LBM_CUDA(h, lbm::launch_sum_partials(scratch, h->P, h->red, h->stream));
       double s = 0.0;
@@ -651,6 +774,7 @@ int lbm_get_state(lbm_handle* h, double* f, int where, int64_t* steps_done) {
   if (!h) { set_err(g_err, "handle is NULL"); return LBM_EINVAL; }
   if (!f || (where != LBM_HOST && where != LBM_DEVICE)) { set_err(h->err, "bad f or where"); return LBM_EINVAL; }
   if (steps_done) *steps_done = h->steps;
+  if (int rc = form_populations(h)) return rc;
   for (int i = 0; i < 9; ++i) {
     const void* plane = static_cast<const char*>(h->f[h->cur]) + size_t(i) * h->N * h->s;
     const double add = kWeights[i] * h->p.rho_ref;
@@ -667,6 +791,9 @@ int lbm_set_state(lbm_handle* h, const double* f, int where, int64_t steps_done)
   lbm::TraceRange trace("lbm_set_state");
   if (!h) { set_err(g_err, "handle is NULL"); return LBM_EINVAL; }
   if (!f || (where != LBM_HOST && where != LBM_DEVICE)) { set_err(h->err, "bad f or where"); return LBM_EINVAL; }
+  h->pop = true;
+  h->mom = false;
+  h->since_io = 0;
   for (int i = 0; i < 9; ++i) {
     void* plane = static_cast<char*>(h->f[h->cur]) + size_t(i) * h->N * h->s;
     const double sub = kWeights[i] * h->p.rho_ref;
@@ -720,6 +847,9 @@ int lbm_set_params(lbm_handle* h, const lbm_params* p) {
     set_err(h->err, "nx, ny, precision, a, b, R, thermal and wall cannot change on a live handle");
     return LBM_EINVAL;
   }
+  // the populations belong to the parameters of the step that made them, and what a Zou-He wall
+  // sends back to those of the step to come
+  if ((rc = leave_moments(h))) return rc;
   const double rho_ref = h->p.rho_ref;
   void* ws = h->p.workspace;
   const uint64_t wsb = h->p.workspace_bytes;
@@ -771,6 +901,7 @@ int lbm_coexistence(double a, double b, double R, double T, double* rho_v, doubl
 int lbm_autotune(lbm_handle* h, int steps, int* variant, double* ms) {
   if (!h) { set_err(g_err, "handle is NULL"); return LBM_EINVAL; }
   if (steps < 1) { set_err(h->err, "steps must be >= 1"); return LBM_EINVAL; }
+  if (int rc0 = leave_moments(h)) return rc0;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   LBM_CUDA(h, cudaEventCreate(&e0));
   cudaError_t ce = cudaEventCreate(&e1);
@@ -792,11 +923,31 @@ int lbm_autotune(lbm_handle* h, int steps, int* variant, double* ms) {
   for (int v = 0; v < lbm::step_num_variants(h->p.precision) && rc == LBM_OK; ++v) {
     lbm::StepTiling t;
     if (plan_tiling(h->p, h->nsm, &t, h->err, v)) continue;
+    // variant 0 is the step on moments where that is used: timed on moments formed in the
+    // spare buffer
+    const bool walk = v == 0 && walk_usable(h);
+    if (walk && (rc = form_moments(h))) break;
     cudaError_t e = cudaSuccess;
-    for (int w = 0; w < 2 && e == cudaSuccess; ++w) e = lbm::launch_step(h->p.precision, lbm::MODE_STEP, t, h->phys, io, h->stream);
+    auto launch = [&](int n) {
+      for (int k = 0; k < n && e == cudaSuccess && rc == LBM_OK; ++k) {
+        if (walk)
+          rc = walk_launch(h);
+        else
+          e = lbm::launch_step(h->p.precision, lbm::MODE_STEP, t, h->phys, io, h->stream);
+      }
+    };
+    launch(2);
     if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-    for (int k = 0; k < steps && e == cudaSuccess; ++k) e = lbm::launch_step(h->p.precision, lbm::MODE_STEP, t, h->phys, io, h->stream);
+    launch(steps);
     if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
+    if (walk) {  // the populations f[cur] are the state still; their sums again
+      h->mom = false;
+      if (rc == LBM_OK) rc = refresh_partials(h);
+      if (rc) break;
+      io.part_in = h->parts[h->pcur];
+      io.npart_in = h->npart;
+      io.part_out = h->parts[1 - h->pcur];
+    }
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float t_ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&t_ms, e0, e1);
@@ -827,6 +978,7 @@ int lbm_set_tiling(lbm_handle* h, int variant) {
   lbm::StepTiling t;
   int rc = plan_tiling(h->p, h->nsm, &t, h->err, variant);
   if (rc) return rc;
+  if ((rc = leave_moments(h))) return rc;
   h->tiling = t;
   h->P = t.nbands * t.nstrips;
   return LBM_OK;

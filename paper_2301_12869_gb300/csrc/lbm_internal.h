@@ -74,6 +74,42 @@ cudaError_t step_prepare(int precision);  // sets the dynamic shared memory limi
 cudaError_t launch_step(int precision, int mode, const StepTiling& t, const StepPhys& ph,
                         const StepIO& io, cudaStream_t stream);
 
+// ---- the step on moments (lbm_walk.cu), for states with every relaxation time 1: three
+// planes real[3][ny][nx] of (drho, j_x, j_y) of the streamed populations
+enum WalkMode : int { WALK_STEP = 0, WALK_POPULATIONS = 1, WALK_MOMENTS = 2 };
+constexpr int kWalkThreadsF = 512, kWalkThreadsD = 256;  // most threads per CTA (FP32, FP64)
+struct WalkTiling {
+  int nx, ny;
+  int seg;               // lanes that walk together: 8, 16 or 32 (the first and last are halo)
+  int band_w, nbands;    // columns a segment owns, bands
+  int strip_h, nstrips;  // rows a segment owns, strips
+  int threads, ctas;
+  int zh;                // Zou-He walls
+  double inv_n_total;    // 1 / nodes: <rho> = (sum of rho) / nodes
+};
+struct WalkIO {
+  const void* min;        // real[3][ny][nx]: M_t (step, moments) or M_(t-1) (populations)
+  void* mout;             // real[3][ny][nx]: M_(t+1) (step), M_t (pull)
+  const void* fin;        // pull: real[9][ny][nx] populations f*_t
+  void* fout;             // populations: real[9][ny][nx]
+  const double* part_in;  // FP64 partial sums of drho over min (pull: of the populations fin)
+  int npart_in;
+  double* part_out;       // the same of mout, one per CTA; only with Eq. Gravity_2
+  const double* mean_in;  // Zou-He with Eq. Gravity_2: <rho> - rho_ref for the collision of min,
+  double* mean_out;       // and the slot of mout's
+  int* status;
+  double *rho_out, *ux_out, *uy_out;  // moments: doubles [y][x] (may be NULL)
+  void *rho_T, *ux_T, *uy_T;          // thermal step: this step's rho, u as reals [y][x]
+  const void* Tfield;     // thermal: real[ny][nx] (NULL: uniform T)
+};
+// the tiling of a lattice on a GPU of nsm SMs; at most max_ctas CTAs (partial sums)
+void plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, WalkTiling* t);
+cudaError_t launch_walk(int precision, int mode, const WalkTiling& t, const StepPhys& ph, const WalkIO& io,
+                        cudaStream_t stream);
+// M_t of the populations f*_t, and its partial sums (one per CTA of the tiling)
+cudaError_t launch_pull(int precision, const WalkTiling& t, const StepPhys& ph, const WalkIO& io, cudaStream_t stream);
+bool unit_relaxation(const StepPhys& p);  // every relaxation time 1
+
 // initial state and the FP64 partial sums of its stored values into part[0..npart)
 cudaError_t launch_init(int precision, const double* rho0, void* f, int nx, int ny, double rho_ref, double* part,
                         int npart, cudaStream_t stream);

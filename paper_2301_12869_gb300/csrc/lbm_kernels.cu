@@ -1019,10 +1019,6 @@ cudaError_t prepare_variant(const VariantD& v) {
   return e;
 }
 
-bool unit_relaxation(const StepPhys& p) {
-  return p.s_e == 1.0 && p.s_vs == 1.0 && p.s_j == 1.0 && p.s_q == 1.0 && p.s_nu == 1.0;
-}
-
 int grid_for(size_t n, int block) {
   size_t g = (n + block - 1) / block;
   if (g > 8192) g = 8192;
@@ -1033,6 +1029,10 @@ int grid_for(size_t n, int block) {
 }  // namespace
 
 // ---------------------------------------------------------------- launch wrappers
+bool unit_relaxation(const StepPhys& p) {
+  return p.s_e == 1.0 && p.s_vs == 1.0 && p.s_j == 1.0 && p.s_q == 1.0 && p.s_nu == 1.0;
+}
+
 int stages(int precision, int variant) {
   return precision == 1 ? kVariantsF[variant].stages : kVariantsD[variant].stages;
 }

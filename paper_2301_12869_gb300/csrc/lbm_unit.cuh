@@ -1,0 +1,156 @@
+// Per-node physics of the step when every relaxation time is 1 (Lambda = I, the paper's
+// setting, Sec. IV), shared by the moment-walk kernels (lbm_walk.cu) and the batched columns
+// (lbm_batch.cu).
+//
+// With Lambda = I, Eq. LBE's collision is m* = m_eq + S~/2 (Eqs. OperatorMRT, LiFS): the
+// post-collision populations depend on the pulled ones only through rho and j. So a node's
+// state can be held as three numbers - drho = rho - rho_ref, j_x, j_y of the streamed
+// populations - instead of nine, and a step is: psi from rho, the Shan-Chen stencil, F and u,
+// the nine post-collision values (in registers), and the three sums of the ones the
+// neighbours send. The collision itself simplifies: with s = u_x g_x + u_y g_y and
+// g = rho u + F, the energy moments are e* = A - 2 drho and eps* = drho - A with
+// A = 3 s + (sigma/(tau - 1/2)) G^2 |S|^2 / 2, p_xx* = u_x g_x - u_y g_y,
+// p_xy* = (u_x g_y + u_y g_x)/2, j* = j + F, q* = -j*. 46 operations a node instead of 78.
+#pragma once
+
+#include "lbm_physics.cuh"
+
+namespace lbm {
+
+template <typename V>
+struct UnitT {
+  PhysT<V> p;
+  V k1, k1R, k2, k3;  // psi^2 = rho (k1 num/om^3 + k2 rho + k3): 2RT/G, 2R/G, -2a/G, -2/(3G)
+  V kS;               // G^2 sigma/(tau - 1/2)/72: the sigma term's share of A/36
+};
+
+template <typename V>
+UnitT<V> to_unit(const StepPhys& s) {
+  UnitT<V> u;
+  u.p = to_phys<V>(s);
+  u.k1 = host_value<V>(2.0 * s.RT / s.G);
+  u.k1R = host_value<V>(2.0 * s.R / s.G);
+  u.k2 = host_value<V>(-2.0 * s.a / s.G);
+  u.k3 = host_value<V>(-2.0 / (3.0 * s.G));
+  u.kS = host_value<V>(s.G * s.G * s.sig_e / 72.0);
+  return u;
+}
+
+// ---- reciprocal and reciprocal square root of a positive normal value
+// FP64: the hardware's 20-bit seed and one Householder step of third order (error of the seed
+// cubed: 2^-57), 3 and 5 FP64 instructions instead of the IEEE division's and square root's
+// 9 and more - GB300 issues an FP64 instruction per SM only every 15 clocks, so the FP64
+// step's time is the count of these. Results are within about 1 ulp.
+__device__ __forceinline__ double unit_rcp(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);  // y (1 + e + e^2)
+}
+__device__ __forceinline__ double unit_rsqrt(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(fma(e, 0.375, 0.5), y * e, y);  // y (1 + e/2 + 3 e^2/8)
+}
+__device__ __forceinline__ f2 unit_rcp(f2 x) { return make_f2(rcp_approx(lo(x)), rcp_approx(hi(x))); }
+
+// psi of Eqs. EOS and InteractionPotential: psi^2 = rho (k1 num/D + k2 rho + k3) with
+// D = (1 - eta)^3; psi^2 < 0 or NaN, or rho <= 0, is non-physical (psi = 0 for the former).
+// FP32 pairs: an approximate reciprocal and square root, without a branch - one would cut the
+// rows of a walk apart for the instruction scheduler.
+__device__ __forceinline__ f2 unit_psi(f2 rho, f2 k1, f2, const UnitT<f2>& k, int& flag) {
+  const f2 one = cst<f2>(1.0);
+  const f2 eta = k.p.b4 * rho;
+  const f2 om = one - eta;
+  const f2 num = fmadd(eta, fmadd(eta, om, one), one);  // 1 + eta + eta^2 - eta^3
+  const f2 q = num * unit_rcp(om * om * om);
+  const f2 p2 = rho * fmadd(k1, q, fmadd(k.k2, rho, k.k3));
+  const float s = lo(p2), t = hi(p2);
+  if (!(s >= 0.f && t >= 0.f && lo(rho) > 0.f && hi(rho) > 0.f)) flag |= STATUS_NONPHYS;
+  return make_f2(sqrt_approx(fmaxf(s, 0.f)), sqrt_approx(fmaxf(t, 0.f)));
+}
+// FP64: with N = rho (k1 num + (k2 rho + k3) D), psi = sqrt(N/D) = N rsqrt(N D): one
+// reciprocal square root in place of a division and a square root. Anything but positive
+// normal N, D and rho takes the general formula.
+__device__ __forceinline__ bool normal_positive(double x) {
+  return unsigned(__double2hiint(x)) - 0x00100000u < 0x7fe00000u;
+}
+__device__ __forceinline__ double unit_psi(double rho, double k1, double RT, const UnitT<double>& k, int& flag) {
+  const double eta = k.p.b4 * rho;
+  const double om = 1.0 - eta;
+  const double num = fma(eta, fma(eta, om, 1.0), 1.0);
+  const double D = om * om * om;
+  const double N = rho * fma(fma(k.k2, rho, k.k3), D, k1 * num);
+  double psi = N * unit_rsqrt(N * D);
+  if (!(normal_positive(N) && normal_positive(D) && normal_positive(rho))) {
+    psi = psi_of<double>(rho, RT, k.p, flag);
+    if (nonpositive(rho)) flag |= STATUS_NONPHYS;
+  }
+  return psi;
+}
+
+// the post-collision values o of a node with moments (dr, jx, jy) before the collision, the
+// potential psi and the stencil sums (Sx, Sy) (zero on wall rows); dmean = <rho> - rho_ref
+template <typename V>
+struct Velocity {
+  V rho, ux, uy;
+};
+// MEAN: the gravity of Eq. Gravity_2 (else Eq. Gravity_1)
+template <bool MEAN, typename V>
+__device__ __forceinline__ Velocity<V> unit_velocity(V dr, V jx, V jy, V psi, V Sx, V Sy, V dmean, const UnitT<V>& k,
+                                                     V& Fx, V& Fy) {
+  const V half = cst<V>(0.5);
+  const V rho = k.p.rho_ref + dr;
+  const V base = MEAN ? (dr - dmean) : rho;
+  const V t = k.p.negG * psi;
+  Fx = fmadd(t, Sx, base * k.p.gx);
+  Fy = fmadd(t, Sy, base * k.p.gy);
+  const V inv = unit_rcp(rho);
+  return {rho, fmadd(half, Fx, jx) * inv, fmadd(half, Fy, jy) * inv};  // Eq. Momentum
+}
+template <bool MEAN, typename V>
+__device__ __forceinline__ Velocity<V> unit_collide(V dr, V jx, V jy, V psi, V Sx, V Sy, V dmean, const UnitT<V>& k,
+                                                    V (&o)[9]) {
+  V Fx, Fy;
+  const Velocity<V> u = unit_velocity<MEAN>(dr, jx, jy, psi, Sx, Sy, dmean, k, Fx, Fy);
+  const V jsx = jx + Fx, jsy = jy + Fy;                       // j*
+  const V hx = fmadd(cst<V>(0.5), Fx, jsx), hy = fmadd(cst<V>(0.5), Fy, jsy);  // rho u + F
+  const V a = u.ux * hx, b = u.uy * hy;
+  const V pq = fmadd(u.ux, hy, u.uy * hx);                    // 2 p_xy*
+  const V S2 = fmadd(Sx, Sx, Sy * Sy);
+  const V A36 = fmadd(cst<V>(1.0 / 12.0), a + b, k.kS * S2);  // A/36
+  const V pxx = a - b;
+  o[0] = fmadd(cst<V>(-8.0), A36, cst<V>(4.0 / 9.0) * dr);
+  const V ba = fmadd(cst<V>(1.0 / 9.0), dr, A36);
+  const V tp = fmadd(cst<V>(0.25), pxx, ba), tm = fmadd(cst<V>(-0.25), pxx, ba);
+  const V third = cst<V>(1.0 / 3.0), mthird = cst<V>(-1.0 / 3.0);
+  o[1] = fmadd(third, jsx, tp);
+  o[3] = fmadd(mthird, jsx, tp);
+  o[2] = fmadd(third, jsy, tm);
+  o[4] = fmadd(mthird, jsy, tm);
+  const V bd = fmadd(cst<V>(1.0 / 36.0), dr, A36);
+  const V up = fmadd(cst<V>(0.125), pq, bd), um = fmadd(cst<V>(-0.125), pq, bd);
+  const V sxy = jsx + jsy, dyx = jsy - jsx;
+  const V tw = cst<V>(1.0 / 12.0), mtw = cst<V>(-1.0 / 12.0);
+  o[5] = fmadd(tw, sxy, up);
+  o[7] = fmadd(mtw, sxy, up);
+  o[6] = fmadd(tw, dyx, um);
+  o[8] = fmadd(mtw, dyx, um);
+  return u;
+}
+
+// Zou-He wall node (Sec. III): K counts the known populations as zou_he() does; the node's
+// density deviation, and j = -F_g/2 so that the velocity vanishes
+template <typename V>
+__device__ __forceinline__ void unit_zou_he(V K, bool bottom, V dmean, const UnitT<V>& k, V& dr, V& jx, V& jy) {
+  const V sg = (bottom ? cst<V>(0.5) : cst<V>(-0.5)) * k.p.gy;
+  const V num = (k.p.form == 2) ? fmadd(sg, dmean, K) : K - sg * k.p.rho_ref;
+  dr = fast_div(num, cst<V>(1.0) + sg);
+  const V base = (k.p.form == 2) ? (dr - dmean) : (k.p.rho_ref + dr);
+  const V mh = cst<V>(-0.5);
+  jx = mh * (base * k.p.gx);
+  jy = mh * (base * k.p.gy);
+}
+
+}  // namespace lbm

@@ -1,0 +1,608 @@
+// The fused D2Q9 step on moments (all relaxation times 1; arXiv 2301.12869, Sec. III, with
+// Lambda = I as in Sec. IV). The physics and why three numbers a node suffice: lbm_unit.cuh.
+//
+// State: M_t = (drho, j_x, j_y) of the streamed populations at time t, three planes [ny][nx].
+// One launch maps M_t to M_(t+1): collide, then stream (pull) - the population step's order
+// started half a step earlier. The populations after t steps are f*_t = collide(M_(t-1)), and
+// the state before the last step stays in the other buffer, so lbm_get_state writes them from
+// there (WALK_POPULATIONS).
+//
+// Bound: 24 B a node and step against the population kernel's 72 B, and 87 operations a node
+// (packed in pairs for FP32) against 146. FP32 is bound by a row's dependency chain with 16
+// warps on an SM, FP64 by the FP64 pipe (an instruction per SM every 15.4 clocks). Measured
+// against the population step: 1024 x 4096 FP32 53.5 -> 22.5 us a step (4.5 TB/s of its own
+// 24 B), 772 x 1003 16.4 -> 5.9, 256 x 768 11.1 -> 5.9; 1024 x 4096 FP64
+// 1291 -> 821 us.
+//
+// Layout: a warp (or a segment of 8 or 16 lanes on narrow lattices) walks a strip of rows
+// upward. A lane holds two columns of a row, an FP32 pair or two FP64 values (two FP32 pairs a
+// lane need 168 registers and leave 12 warps an SM: 23.7 us); the first and last lane
+// of a segment are halo (x periodic: a lane's columns are taken modulo nx, which its width
+// divides). x neighbours come from the adjacent lane by one shuffle a quantity, y neighbours
+// from a three-row window in registers, so there is no shared memory and no barrier in the
+// walk. At input row q: psi of row q; collision of row q - 1; row q - 2 receives its last
+// contributions and is stored. Of the nine post-collision values the walk keeps column sums
+// only: for target row y
+//   V = f0(y) + f2(y-1) + f4(y+1)                                     (from x)
+//   P = f1(y) + f5(y-1) + f8(y+1),  D = f5(y-1) - f8(y+1)             (from x - 1)
+//   Q = f3(y) + f6(y-1) + f7(y+1),  E = f6(y-1) - f7(y+1)             (from x + 1)
+// so drho = V + P + Q, j_x = P - Q, j_y = f2(y-1) - f4(y+1) + D + E: four shuffled values
+// instead of six. The row loop runs three rows an iteration so that the windows rotate by
+// register renaming; rows are loaded three ahead.
+#include "lbm_dd.cuh"
+#include "lbm_internal.h"
+#include "lbm_ptx.cuh"
+#include "lbm_unit.cuh"
+
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+
+namespace lbm {
+namespace {
+
+// ---- the columns of a row that a lane holds: N values (FP32 pairs, or FP64 columns)
+template <typename T>
+struct LaneOf;
+template <>
+struct LaneOf<float> {
+  using V = f2;
+  static constexpr int N = 1;
+};
+template <>
+struct LaneOf<double> {
+  using V = double;
+  static constexpr int N = 2;
+};
+template <typename V, int N>
+struct Lane {
+  V v[N];
+};
+template <typename T>
+using LaneT = Lane<typename LaneOf<T>::V, LaneOf<T>::N>;
+template <typename T>
+constexpr int kColumns = LaneOf<T>::N* VecTraits<typename LaneOf<T>::V>::width;  // a lane's columns
+
+__device__ __forceinline__ Lane<f2, 1> load_lane(const float* p) {
+  return {{*reinterpret_cast<const f2*>(p)}};
+}
+__device__ __forceinline__ Lane<double, 2> load_lane(const double* p) {
+  const double2 q = *reinterpret_cast<const double2*>(p);
+  return {{q.x, q.y}};
+}
+__device__ __forceinline__ void store_lane(float* p, const Lane<f2, 1>& q) {
+  *reinterpret_cast<f2*>(p) = q.v[0];
+}
+__device__ __forceinline__ void store_lane(double* p, const Lane<double, 2>& q) {
+  *reinterpret_cast<double2*>(p) = make_double2(q.v[0], q.v[1]);
+}
+// into a caller's array of doubles, which may start on any 8-byte boundary
+__device__ __forceinline__ void store_doubles(double* p, const Lane<double, 2>& q) {
+  if (reinterpret_cast<uintptr_t>(p) & 15u) {
+    p[0] = q.v[0];
+    p[1] = q.v[1];
+  } else {
+    store_lane(p, q);
+  }
+}
+template <int N>
+__device__ __forceinline__ void store_doubles(double* p, const Lane<f2, N>& q) {
+#pragma unroll
+  for (int j = 0; j < N; ++j) store_doubles(p + 2 * j, Lane<double, 2>{{lo(q.v[j]), hi(q.v[j])}});
+}
+
+// value at x - 1 / x + 1 of every column; the segment's edge lanes get their own value there
+template <int N>
+__device__ __forceinline__ Lane<f2, N> from_left(const Lane<f2, N>& q, int seg) {
+  Lane<f2, N> o;
+  o.v[0] = make_f2(__shfl_up_sync(0xffffffffu, hi(q.v[N - 1]), 1, seg), lo(q.v[0]));
+#pragma unroll
+  for (int j = 1; j < N; ++j) o.v[j] = make_f2(hi(q.v[j - 1]), lo(q.v[j]));
+  return o;
+}
+template <int N>
+__device__ __forceinline__ Lane<f2, N> from_right(const Lane<f2, N>& q, int seg) {
+  Lane<f2, N> o;
+  o.v[N - 1] = make_f2(hi(q.v[N - 1]), __shfl_down_sync(0xffffffffu, lo(q.v[0]), 1, seg));
+#pragma unroll
+  for (int j = 0; j + 1 < N; ++j) o.v[j] = make_f2(hi(q.v[j]), lo(q.v[j + 1]));
+  return o;
+}
+template <int N>
+__device__ __forceinline__ Lane<double, N> from_left(const Lane<double, N>& q, int seg) {
+  Lane<double, N> o;
+  o.v[0] = __shfl_up_sync(0xffffffffu, q.v[N - 1], 1, seg);
+#pragma unroll
+  for (int j = 1; j < N; ++j) o.v[j] = q.v[j - 1];
+  return o;
+}
+template <int N>
+__device__ __forceinline__ Lane<double, N> from_right(const Lane<double, N>& q, int seg) {
+  Lane<double, N> o;
+  o.v[N - 1] = __shfl_down_sync(0xffffffffu, q.v[0], 1, seg);
+#pragma unroll
+  for (int j = 0; j + 1 < N; ++j) o.v[j] = q.v[j + 1];
+  return o;
+}
+
+template <typename V, int N>
+__device__ __forceinline__ Lane<V, N> operator+(const Lane<V, N>& x, const Lane<V, N>& y) {
+  Lane<V, N> o;
+#pragma unroll
+  for (int j = 0; j < N; ++j) o.v[j] = x.v[j] + y.v[j];
+  return o;
+}
+template <typename V, int N>
+__device__ __forceinline__ Lane<V, N> operator-(const Lane<V, N>& x, const Lane<V, N>& y) {
+  Lane<V, N> o;
+#pragma unroll
+  for (int j = 0; j < N; ++j) o.v[j] = x.v[j] - y.v[j];
+  return o;
+}
+template <typename V, int N>
+__device__ __forceinline__ Lane<V, N> operator*(V s, const Lane<V, N>& x) {
+  Lane<V, N> o;
+#pragma unroll
+  for (int j = 0; j < N; ++j) o.v[j] = s * x.v[j];
+  return o;
+}
+template <typename V, int N>
+__device__ __forceinline__ Lane<V, N> fma_lane(V s, const Lane<V, N>& x, const Lane<V, N>& y) {
+  Lane<V, N> o;
+#pragma unroll
+  for (int j = 0; j < N; ++j) o.v[j] = fmadd(s, x.v[j], y.v[j]);
+  return o;
+}
+template <typename V, int N>
+__device__ __forceinline__ V sum_lane(const Lane<V, N>& x) {
+  V o = x.v[0];
+#pragma unroll
+  for (int j = 1; j < N; ++j) o = o + x.v[j];
+  return o;
+}
+template <typename V, int N>
+__device__ __forceinline__ Lane<V, N> splat_lane(V s) {
+  Lane<V, N> o;
+#pragma unroll
+  for (int j = 0; j < N; ++j) o.v[j] = s;
+  return o;
+}
+
+// sum over the warp of the lanes' mass partials, in every lane: the FP32 accumulators' two-sum
+// pairs are added as pairs (48 bits), since FP64 conversions and additions issue at 1/64 of
+// the FP32 rate
+__device__ __forceinline__ double warp_total(double s) { return warp_sum(s); }
+__device__ __forceinline__ dd warp_total(dd s) {
+#pragma unroll
+  for (int m = 16; m; m >>= 1)
+    s = s + dd{__shfl_xor_sync(0xffffffffu, s.hi, m), __shfl_xor_sync(0xffffffffu, s.lo, m)};
+  return s;
+}
+__device__ __forceinline__ double lane_mass(const Acc<double>& a) { return a.value(); }
+__device__ __forceinline__ dd lane_mass(const Acc<f2>& a) {
+  return dd{lo(a.hi[0]), lo(a.lo[0])} + dd{hi(a.hi[0]), hi(a.lo[0])};
+}
+// the CTA's total into out[blockIdx.x]; red: one value a warp
+template <typename V, typename S>
+__device__ __forceinline__ void cta_mass(const Acc<V>& acc, S* red, double* out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const S v = warp_total(lane_mass(acc));
+  if (lane == 0) red[warp] = v;
+  __syncthreads();
+  if (warp == 0) {
+    const S t = warp_total(lane < int(blockDim.x >> 5) ? red[lane] : S{});
+    if (lane == 0) out[blockIdx.x] = hsum(t);
+  }
+}
+template <typename V>
+using MassOf = decltype(lane_mass(Acc<V>{}));
+
+template <typename T, int MODE, bool TH, bool MEAN>
+__global__ void __launch_bounds__(sizeof(T) == 4 ? kWalkThreadsF : kWalkThreadsD, 1)
+    walk_kernel(const WalkTiling tl, const UnitT<typename LaneOf<T>::V> k, const WalkIO io) {
+  using V = typename LaneOf<T>::V;
+  using L = LaneT<T>;
+  constexpr int N = LaneOf<T>::N, W = kColumns<T>;
+  constexpr int HALO = MODE == WALK_STEP ? 2 : 1;  // rows read beyond the strip on each side
+  __shared__ double mean_s[2];
+  __shared__ MassOf<V> sums[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nx = tl.nx, ny = tl.ny, seg = tl.seg;
+  // this segment's band and strip; segments past the last strip own nothing (they stay with
+  // their warp for its shuffles)
+  const int item = (blockIdx.x * blockDim.x + tid) / seg;
+  const int l = tid & (seg - 1);
+  const int band = item % tl.nbands, strip = item / tl.nbands;
+  const int ya = strip * tl.strip_h, yb = min(ya + tl.strip_h, ny);
+  const int c0 = band * tl.band_w + (l - 1) * W;  // first column, unwrapped
+  const bool own = l >= 1 && l < seg - 1 && c0 < min(band * tl.band_w + tl.band_w, nx);
+  int x = c0 % nx;
+  if (x < 0) x += nx;
+  const size_t plane = size_t(nx) * ny;
+  const T* mdr = static_cast<const T*>(io.min) + x;
+  const T* Tf = TH ? static_cast<const T*>(io.Tfield) + x : nullptr;
+  const bool zh = tl.zh != 0;
+  griddep_wait();  // launched as a dependent of the previous kernel: its state is complete
+  griddep_launch_dependents();
+
+  struct Raw {
+    L dr, jx, jy, t;
+  };
+  // rows beyond the strip's reach or the lattice load the nearest one that is not: what is
+  // formed from them is never used
+  const int q_top = min(yb + HALO, ny) - 1;
+  auto fetch = [&](int q, Raw& w) {
+    const size_t n = size_t(max(min(q, q_top), 0)) * nx;
+    w.dr = load_lane(mdr + n);
+    w.jx = load_lane(mdr + plane + n);
+    w.jy = load_lane(mdr + 2 * plane + n);
+    if constexpr (TH) w.t = load_lane(Tf + n);
+  };
+  const int q0 = ya - HALO;
+  Raw r0, r1, r2;
+  fetch(q0, r0);
+  fetch(q0 + 1, r1);
+  fetch(q0 + 2, r2);
+
+  // <rho> - rho_ref for the collision, and with Zou-He walls the one of the closure (the mass
+  // of the populations about to be streamed = the sum of drho now, since the collision keeps
+  // it). One warp of the CTA sums while the others form psi of their first rows.
+  const V zero = cst<V>(0.0);
+  const L zero2 = splat_lane<V, N>(zero);
+  V dmean = zero, dclose = zero;
+  if (MEAN && warp == 0) {
+    const double s = warp_sum_partials(io.part_in, io.npart_in);
+    if (lane == 0) {
+      const double m = s * tl.inv_n_total;
+      mean_s[0] = m;
+      mean_s[1] = zh ? *io.mean_in : m;
+      if (MODE == WALK_STEP && zh && blockIdx.x == 0) *io.mean_out = m;
+    }
+  }
+  auto wait_mean = [&] {
+    if (MEAN) {
+      __syncthreads();
+      dclose = cst<V>(mean_s[0]);
+      dmean = cst<V>(mean_s[1]);
+    }
+  };
+
+  int flag = 0;
+  Acc<V> acc;
+  // psi of row q - 1; (1/12) d of row q - 1, (1/3) d(q - 1) + (1/12) d(q - 2), and
+  // (1/3) psi + (1/12) s of rows q - 2, q - 1 (d, s: psi(x+1) -+ psi(x-1))
+  L psi1 = zero2, A1 = zero2, X1 = zero2, B0 = zero2, B1 = zero2;
+  L dr1 = zero2, jx1 = zero2, jy1 = zero2;  // moments of row q - 1
+  L V1 = zero2, P1 = zero2, Q1 = zero2;     // f2, f5, f6 of row q - 2 (for target q - 1)
+  // target q - 2 so far: sums from rows q-3 and q-2, its southern f2, f5, f6, and what the
+  // bottom wall sends back without an x shift
+  L S2 = zero2, P2 = zero2, Q2 = zero2, a2 = zero2, a5 = zero2, a6 = zero2, Jh = zero2;
+  const V c13 = cst<V>(1.0 / 3.0), c112 = cst<V>(1.0 / 12.0);
+
+  // EDGE: rows at the walls or beyond may take part
+  auto body = [&](int q, Raw& in, auto edge) {
+    constexpr bool EDGE = decltype(edge)::value;
+    // ---- psi of row q
+    const L dr2 = in.dr, jx2 = in.jx, jy2 = in.jy;
+    L psi2;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      if constexpr (TH)
+        psi2.v[j] = unit_psi(k.p.rho_ref + dr2.v[j], k.k1R * in.t.v[j], k.p.R * in.t.v[j], k, flag);
+      else
+        psi2.v[j] = unit_psi(k.p.rho_ref + dr2.v[j], k.k1, k.p.RT, k, flag);
+    }
+    fetch(q + 3, in);
+    const L w = from_left(psi2, seg), e = from_right(psi2, seg);
+    const L d2 = e - w;
+    const L A2 = c112 * d2;
+    const L B2 = fma_lane(c13, psi2, c112 * (e + w));
+    // ---- collision of row r = q - 1 (Eq. ShanChenForce stencil; zero on the wall rows)
+    const int r = q - 1;
+    L Sx = X1 + A2, Sy = B2 - B0;
+    if (EDGE && (r <= 0 || r >= ny - 1)) Sx = Sy = zero2;
+    X1 = fma_lane(c13, d2, A1);
+    A1 = A2;
+    B0 = B1;
+    B1 = B2;
+    L rho, ux, uy;
+    if constexpr (MODE == WALK_MOMENTS) {
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        V Fx, Fy;
+        const Velocity<V> u =
+            unit_velocity<MEAN>(dr1.v[j], jx1.v[j], jy1.v[j], psi1.v[j], Sx.v[j], Sy.v[j], dmean, k, Fx, Fy);
+        rho.v[j] = u.rho;
+        ux.v[j] = u.ux;
+        uy.v[j] = u.uy;
+      }
+      if (own && r >= ya && r < yb) {
+        const size_t n = size_t(r) * nx + x;
+        if (io.rho_out) store_doubles(io.rho_out + n, rho);
+        if (io.ux_out) store_doubles(io.ux_out + n, ux);
+        if (io.uy_out) store_doubles(io.uy_out + n, uy);
+      }
+    } else {
+      L f[9];
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        V o[9];
+        const Velocity<V> u =
+            unit_collide<MEAN>(dr1.v[j], jx1.v[j], jy1.v[j], psi1.v[j], Sx.v[j], Sy.v[j], dmean, k, o);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i].v[j] = o[i];
+        rho.v[j] = u.rho;
+        ux.v[j] = u.ux;
+        uy.v[j] = u.uy;
+      }
+      if constexpr (MODE == WALK_POPULATIONS) {
+        if (own && r >= ya && r < yb) {
+          T* dst = static_cast<T*>(io.fout) + size_t(r) * nx + x;
+#pragma unroll
+          for (int i = 0; i < 9; ++i) store_lane(dst + i * plane, f[i]);
+        }
+      } else {
+        if (TH && own && r >= ya && r < yb) {  // this step's rho, u for the energy equation
+          const size_t n = size_t(r) * nx + x;
+          store_lane(static_cast<T*>(io.rho_T) + n, rho);
+          store_lane(static_cast<T*>(io.ux_T) + n, ux);
+          store_lane(static_cast<T*>(io.uy_T) + n, uy);
+        }
+        // ---- target y = q - 2 receives row r's f4, f8, f7; past the top wall row (r = ny) row
+        // ny - 1's own f2, f5, f6 come back instead (halfway bounce-back)
+        const int y = r - 1;
+        L n4 = f[4], n8 = f[8], n7 = f[7];
+        if (EDGE && r == ny) {
+          n4 = n8 = n7 = zero2;
+          if (!zh) {
+            n4 = V1 + (P1 + Q1);
+            Jh = Jh + (Q1 - P1);
+          }
+        }
+        const L Ps = from_left(P2 + n8, seg), Ds = from_left(a5 - n8, seg);
+        const L Qs = from_right(Q2 + n7, seg), Es = from_right(a6 - n7, seg);
+        L dr = (S2 + n4) + (Ps + Qs);
+        L jx = Ps - Qs;
+        L jy = (a2 - n4) + (Ds + Es);
+        if (EDGE && (y == 0 || y == ny - 1)) {
+          jx = jx + Jh;
+          if (zh) {
+            const L K = y == 0 ? dr - jy : dr + jy;
+#pragma unroll
+            for (int j = 0; j < N; ++j) unit_zou_he(K.v[j], y == 0, dclose, k, dr.v[j], jx.v[j], jy.v[j]);
+          }
+        }
+        if (own && y >= ya && y < yb) {
+          T* dst = static_cast<T*>(io.mout) + size_t(y) * nx + x;
+          store_lane(dst, dr);
+          store_lane(dst + plane, jx);
+          store_lane(dst + 2 * plane, jy);
+          if (MEAN) acc.add(sum_lane(dr));
+        }
+        // ---- target r: its own f0, f1, f3 on top of row r - 1's f2, f5, f6; at the bottom wall
+        // its f4, f7, f8 come back (Zou-He: the closure replaces them)
+        a2 = V1;
+        a5 = P1;
+        a6 = Q1;
+        if (EDGE) Jh = zero2;
+        if (EDGE && r == 0) {
+          a2 = a5 = a6 = zero2;
+          if (!zh) {
+            a2 = f[4] + (f[7] + f[8]);
+            Jh = f[7] - f[8];
+          }
+        }
+        S2 = a2 + f[0];
+        P2 = a5 + f[1];
+        Q2 = a6 + f[3];
+        V1 = f[2];
+        P1 = f[5];
+        Q1 = f[6];
+      }
+    }
+    dr1 = dr2;
+    jx1 = jx2;
+    jy1 = jy2;
+    psi1 = psi2;
+  };
+  // input rows ya - HALO .. yb + HALO - 1 (a step stores row yb - 1 at q = yb + 1), three at a
+  // time; away from the walls without their cases (uniform over the warp)
+  const int nq = tl.strip_h + 2 * HALO;
+  body(q0, r0, std::true_type{});  // psi only: no row below to collide
+  if (MODE != WALK_STEP) wait_mean();
+  body(q0 + 1, r1, std::true_type{});
+  if (MODE == WALK_STEP) wait_mean();
+  body(q0 + 2, r2, std::true_type{});
+  for (int it = 3; it < nq; it += 3) {
+    const int q = q0 + it;
+    if (MODE == WALK_STEP && __all_sync(0xffffffffu, q >= 3 && q + 2 < ny)) {
+      body(q, r0, std::false_type{});
+      body(q + 1, r1, std::false_type{});
+      body(q + 2, r2, std::false_type{});
+    } else {
+      body(q, r0, std::true_type{});
+      body(q + 1, r1, std::true_type{});
+      body(q + 2, r2, std::true_type{});
+    }
+  }
+
+  const int wf = __reduce_or_sync(0xffffffffu, flag);
+  if (lane == 0 && wf) atomicOr(io.status, wf);
+  if (MODE == WALK_STEP && MEAN) {
+    cta_mass(acc, sums, io.part_out);
+  }
+}
+
+// a lane's columns of a row at x, each with its neighbour at x - 1 (LEFT) or x + 1 instead;
+// xn: the neighbour beyond the lane's columns
+template <bool LEFT>
+__device__ __forceinline__ Lane<f2, 1> shift(const float* p, int x, int xn, std::bool_constant<LEFT>) {
+  const Lane<f2, 1> c = load_lane(p + x);
+  if (LEFT) return {{make_f2(p[xn], lo(c.v[0]))}};
+  return {{make_f2(hi(c.v[0]), p[xn])}};
+}
+template <bool LEFT>
+__device__ __forceinline__ Lane<double, 2> shift(const double* p, int x, int xn, std::bool_constant<LEFT>) {
+  const Lane<double, 2> c = load_lane(p + x);
+  if (LEFT) return {{p[xn], c.v[0]}};
+  return {{c.v[1], p[xn]}};
+}
+
+// ---- populations -> moments: M_t of the stored f*_t (Eqs. LBE, Density, Momentum without the
+// force), and its FP64 partial sums; one thread a group of 16 bytes of a row
+template <typename T>
+__global__ void __launch_bounds__(256) pull_kernel(const WalkTiling tl, const UnitT<typename LaneOf<T>::V> k,
+                                                   const WalkIO io) {
+  using V = typename LaneOf<T>::V;
+  using L = LaneT<T>;
+  constexpr int N = LaneOf<T>::N, W = kColumns<T>;
+  __shared__ double mean_s;
+  __shared__ MassOf<V> sums[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nx = tl.nx, ny = tl.ny, groups = nx / W;
+  const size_t plane = size_t(nx) * ny;
+  const T* f = static_cast<const T*>(io.fin);
+  const bool zh = tl.zh != 0;
+  V dclose = cst<V>(0.0);
+  if (k.p.form == 2 && zh) {  // <rho> of the closure: the stored populations' mass
+    if (warp == 0) {
+      const double s = warp_sum_partials(io.part_in, io.npart_in);
+      if (lane == 0) {
+        mean_s = s * tl.inv_n_total;
+        if (blockIdx.x == 0) *io.mean_out = mean_s;
+      }
+    }
+    __syncthreads();
+    dclose = cst<V>(mean_s);
+  }
+  Acc<V> acc;
+  const size_t total = size_t(groups) * ny;
+  for (size_t g = blockIdx.x * size_t(blockDim.x) + tid; g < total; g += size_t(gridDim.x) * blockDim.x) {
+    const int y = int(g / groups), x = int(g - size_t(y) * groups) * W;
+    const int xl = x == 0 ? nx - 1 : x - 1, xr = x + W == nx ? 0 : x + W;
+    auto at = [&](int i, int row) { return f + i * plane + size_t(row) * nx; };
+    auto centre = [&](int i, int row) { return load_lane(at(i, row) + x); };
+    auto west = [&](int i, int row) { return shift(at(i, row), x, xl, std::true_type{}); };
+    auto east = [&](int i, int row) { return shift(at(i, row), x, xr, std::false_type{}); };
+    const bool lo_w = y == 0, hi_w = y == ny - 1;
+    const L f0 = centre(0, y), f1 = west(1, y), f3 = east(3, y);
+    const L f2_ = lo_w ? centre(4, y) : centre(2, y - 1);
+    const L f5 = lo_w ? centre(7, y) : west(5, y - 1);
+    const L f6 = lo_w ? centre(8, y) : east(6, y - 1);
+    const L f4 = hi_w ? centre(2, y) : centre(4, y + 1);
+    const L f7 = hi_w ? centre(5, y) : east(7, y + 1);
+    const L f8 = hi_w ? centre(6, y) : west(8, y + 1);
+    const L P = (f1 + f5) + f8, Q = (f3 + f6) + f7;
+    L dr = ((f0 + f2_) + f4) + (P + Q);
+    L jx = P - Q;
+    L jy = (f2_ - f4) + ((f5 - f8) + (f6 - f7));
+    if (zh && (lo_w || hi_w)) {
+      const L K = lo_w ? (f0 + (f1 + f3)) + cst<V>(2.0) * (f4 + (f7 + f8))
+                            : (f0 + (f1 + f3)) + cst<V>(2.0) * (f2_ + (f5 + f6));
+#pragma unroll
+      for (int j = 0; j < N; ++j) unit_zou_he(K.v[j], lo_w, dclose, k, dr.v[j], jx.v[j], jy.v[j]);
+    }
+    T* dst = static_cast<T*>(io.mout) + size_t(y) * nx + x;
+    store_lane(dst, dr);
+    store_lane(dst + plane, jx);
+    store_lane(dst + 2 * plane, jy);
+    acc.add(sum_lane(dr));
+  }
+  if (k.p.form == 2) {
+    cta_mass(acc, sums, io.part_out);
+  }
+}
+
+}  // namespace
+
+// The band layout (8, 16 or 32 lanes a segment) that wastes the fewest halo lanes, and the strip
+// height with the smallest estimated time. A wave of warps takes t0 + rows x (time of a row with
+// w warps on an SM): measured for FP32 0.22 us a row with 2 warps (its latency), 0.30 with 8,
+// 0.50 with 16; an FP64 row is bound by the SM's FP64 pipe (1.57 us a warp: 100 issue slots of
+// 15.4 clocks a column) and takes 5 us alone. 1024 x 4096 FP32: 31-row strips, one wave of
+// 16 warps per SM, 22.5 us; 30 rows (two waves) 41 us, 50 rows (10 warps per SM) 27.6 us.
+void plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, WalkTiling* t) {
+  const bool fp32 = precision == 1;
+  const int W = fp32 ? kColumns<float> : kColumns<double>;
+  t->nx = nx;
+  t->ny = ny;
+  t->zh = zh ? 1 : 0;
+  t->inv_n_total = 1.0 / (double(nx) * double(ny));
+  long best_lanes = 0;
+  for (int seg : {32, 16, 8}) {
+    const int own = (seg - 2) * W;
+    const int nb = (nx + own - 1) / own;
+    if (best_lanes == 0 || long(nb) * seg < best_lanes) {
+      best_lanes = long(nb) * seg;
+      t->seg = seg;
+      t->nbands = nb;
+    }
+  }
+  t->band_w = ((nx + t->nbands - 1) / t->nbands + W - 1) / W * W;
+  t->nbands = (nx + t->band_w - 1) / t->band_w;
+  const int most_warps = (fp32 ? kWalkThreadsF : kWalkThreadsD) / 32;
+  auto set_rows = [&](int h) {
+    t->strip_h = h;
+    t->nstrips = (ny + h - 1) / h;
+    const long warps = (long(t->nstrips) * t->nbands * t->seg + 31) / 32;
+    const int per_cta = int(std::min<long>(most_warps, (warps + nsm - 1) / nsm));
+    t->threads = 32 * per_cta;
+    t->ctas = int((warps + per_cta - 1) / per_cta);
+    return warps;
+  };
+  double best = 0.0;
+  int best_h = 1;
+  for (int h = 1; h <= ny; h = h < 32 ? h + 1 : h + h / 16) {
+    const long per_sm = (set_rows(h) + nsm - 1) / nsm;
+    const double waves = double((per_sm + most_warps - 1) / most_warps);
+    const double w = double(std::min<long>(per_sm, most_warps));
+    const double row = fp32 ? 0.18 + 0.02 * w : std::max(5.0, 1.57 * w);
+    const double time = waves * (1.4 + (h + 6) / 3 * 3 * row);
+    if (best == 0.0 || time < best) {
+      best = time;
+      best_h = h;
+    }
+  }
+  set_rows(best_h);
+  // the partial sums' slots bound the grid
+  while (t->ctas > max_ctas && t->strip_h < ny) set_rows(std::min(ny, t->strip_h + std::max(1, t->strip_h / 8)));
+}
+
+namespace {
+template <typename T, int MODE, bool TH>
+cudaError_t launch_walk_m(const WalkTiling& t, const StepPhys& ph, const WalkIO& io, cudaStream_t s) {
+  const auto k = to_unit<typename LaneOf<T>::V>(ph);
+  return ph.form == 2 ? launch_dependent(walk_kernel<T, MODE, TH, true>, dim3(t.ctas), dim3(t.threads), 0, s, t, k, io)
+                      : launch_dependent(walk_kernel<T, MODE, TH, false>, dim3(t.ctas), dim3(t.threads), 0, s, t, k, io);
+}
+template <typename T>
+cudaError_t launch_walk_t(int mode, const WalkTiling& t, const StepPhys& ph, const WalkIO& io, cudaStream_t s) {
+  const bool th = io.Tfield != nullptr;
+  if (mode == WALK_STEP)
+    return th ? launch_walk_m<T, WALK_STEP, true>(t, ph, io, s) : launch_walk_m<T, WALK_STEP, false>(t, ph, io, s);
+  if (mode == WALK_POPULATIONS)
+    return th ? launch_walk_m<T, WALK_POPULATIONS, true>(t, ph, io, s)
+              : launch_walk_m<T, WALK_POPULATIONS, false>(t, ph, io, s);
+  return th ? launch_walk_m<T, WALK_MOMENTS, true>(t, ph, io, s) : launch_walk_m<T, WALK_MOMENTS, false>(t, ph, io, s);
+}
+}  // namespace
+
+cudaError_t launch_walk(int precision, int mode, const WalkTiling& t, const StepPhys& ph, const WalkIO& io,
+                        cudaStream_t stream) {
+  // a thermal step stores its rho, u: refuse a launch without somewhere to put them
+  if (io.Tfield && mode == WALK_STEP && !(io.rho_T && io.ux_T && io.uy_T)) return cudaErrorInvalidValue;
+  return precision == 1 ? launch_walk_t<float>(mode, t, ph, io, stream)
+                        : launch_walk_t<double>(mode, t, ph, io, stream);
+}
+
+cudaError_t launch_pull(int precision, const WalkTiling& t, const StepPhys& ph, const WalkIO& io, cudaStream_t stream) {
+  if (precision == 1)
+    pull_kernel<float><<<t.ctas, 256, 0, stream>>>(t, to_unit<f2>(ph), io);
+  else
+    pull_kernel<double><<<t.ctas, 256, 0, stream>>>(t, to_unit<double>(ph), io);
+  return cudaGetLastError();
+}
+
+}  // namespace lbm
