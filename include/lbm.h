@@ -262,13 +262,16 @@ int lbm_batch_run_stall(lbm_batch* b, double tol, int64_t max_steps, int check_e
  * (c_4 = 1) minimising |sum_j c_j (x_{j+1} - x_j)| weight sum_j c_j x_j / sum_j c_j - which
  * captures the damped oscillations in which the columns' slow modes decay. The estimate
  * replaces the state when every density stays positive, and is undone when the next
- * residual check is worse than the one before it. checks = 0 turns it off. The library
+ * residual check is worse than the one before it (x: the populations, or with every
+ * relaxation time 1 the moments rho, j of the streamed ones, which determine them; no estimate
+ * is taken at a run's last step). checks = 0 turns it off. The library
  * allocates 6 x 9 x (total nodes) reals once. Not carried over by lbm_batch_convert. */
 int lbm_batch_set_acceleration(lbm_batch* b, int checks);
 
 /* Block size of the batched kernel (a runtime choice, no counterpart in the paper): threads
- * = 128, 256 (the default) or 512 per CTA; a CTA iterates one column at a time. Carried
- * over by lbm_batch_convert. LBM_EINVAL for another value. */
+ * = 128, 256 (the default) or 512 per CTA; a CTA iterates one column at a time. Columns that are
+ * iterated on chip (every relaxation time 1, rows of up to 32 threads) have a block size by their
+ * height instead. Carried over by lbm_batch_convert. LBM_EINVAL for another value. */
 int lbm_batch_set_threads(lbm_batch* b, int threads);
 /* Autotuner of the batched kernel's block size: on a copy of the batch's current state,
  * every column runs `steps` (>= 1) steps with no residual stop (after a 2-step warm-up) for

@@ -13,6 +13,7 @@
 // p_xy* = (u_x g_y + u_y g_x)/2, j* = j + F, q* = -j*. 46 operations a node instead of 78.
 #pragma once
 
+#include "lbm_dd.cuh"
 #include "lbm_physics.cuh"
 
 namespace lbm {
@@ -36,6 +37,24 @@ UnitT<V> to_unit(const StepPhys& s) {
   return u;
 }
 
+// c x for a power of two c, and c x + y: exact scalings, which cost a double-float value two
+// multiplications instead of a product; y + c x and y - c x (one product for double-float)
+template <typename V>
+__device__ __forceinline__ V scale2(double c, V x) {
+  return cst<V>(c) * x;
+}
+__device__ __forceinline__ dd scale2(double c, dd x) { return dd{float(c) * x.hi, float(c) * x.lo}; }
+template <typename V>
+__device__ __forceinline__ V fma2(double c, V x, V y) {
+  return fmadd(cst<V>(c), x, y);
+}
+__device__ __forceinline__ dd fma2(double c, dd x, dd y) { return scale2(c, x) + y; }
+template <typename V>
+__device__ __forceinline__ void plus_minus(double c, V x, V y, V& p, V& m) {
+  p = fmadd(cst<V>(c), x, y);
+  m = fmadd(cst<V>(-c), x, y);
+}
+
 // ---- reciprocal and reciprocal square root of a positive normal value
 // FP64: the hardware's 20-bit seed and one Householder step of third order (error of the seed
 // cubed: 2^-57), 3 and 5 FP64 instructions instead of the IEEE division's and square root's
@@ -54,6 +73,24 @@ __device__ __forceinline__ double unit_rsqrt(double x) {
   return fma(fma(e, 0.375, 0.5), y * e, y);  // y (1 + e/2 + 3 e^2/8)
 }
 __device__ __forceinline__ f2 unit_rcp(f2 x) { return make_f2(rcp_approx(lo(x)), rcp_approx(hi(x))); }
+
+// double-float: an FP32 guess (refined to 2^-23), whose correction is formed in FP32 from the
+// exact remainder, so the result is good to about 2^-46
+__device__ __forceinline__ dd unit_rcp(dd x) {
+  float y = rcp_approx(x.hi);
+  y = __fmaf_rn(y, __fmaf_rn(-x.hi, y, 1.f), y);
+  const float e = __fmaf_rn(-x.lo, y, __fmaf_rn(-x.hi, y, 1.f));
+  return dd_fast_two_sum(y, __fmul_rn(y, __fmaf_rn(e, e, e)));
+}
+__device__ __forceinline__ dd unit_rsqrt(dd x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x.hi));
+  y = __fmaf_rn(__fmul_rn(0.5f, y), __fmaf_rn(-__fmul_rn(x.hi, y), y, 1.f), y);
+  const dd y2 = dd_two_prod(y, y);
+  const dd t = x * y2;                               // 1 - e
+  const float e = __fsub_rn(__fsub_rn(1.f, t.hi), t.lo);
+  return dd_fast_two_sum(y, __fmul_rn(__fmul_rn(y, e), __fmaf_rn(0.375f, e, 0.5f)));
+}
 
 // psi of Eqs. EOS and InteractionPotential: psi^2 = rho (k1 num/D + k2 rho + k3) with
 // D = (1 - eta)^3; psi^2 < 0 or NaN, or rho <= 0, is non-physical (psi = 0 for the former).
@@ -90,53 +127,81 @@ __device__ __forceinline__ double unit_psi(double rho, double k1, double RT, con
   return psi;
 }
 
+__device__ __forceinline__ dd unit_psi(dd rho, dd k1, dd RT, const UnitT<dd>& k, int& flag) {
+  const dd one = cst<dd>(1.0);
+  const dd eta = k.p.b4 * rho;
+  const dd om = one - eta;
+  const dd num = fmadd(eta, fmadd(eta, om, one), one);
+  const dd D = om * om * om;
+  const dd N = rho * fmadd(fmadd(k.k2, rho, k.k3), D, k1 * num);
+  if (N.hi > 0.f && D.hi > 0.f && rho.hi > 0.f) return N * unit_rsqrt(N * D);
+  if (nonpositive(rho)) flag |= STATUS_NONPHYS;
+  return psi_of<dd>(rho, RT, k.p, flag);
+}
+
 // the post-collision values o of a node with moments (dr, jx, jy) before the collision, the
 // potential psi and the stencil sums (Sx, Sy) (zero on wall rows); dmean = <rho> - rho_ref
 template <typename V>
 struct Velocity {
   V rho, ux, uy;
 };
-// MEAN: the gravity of Eq. Gravity_2 (else Eq. Gravity_1)
-template <bool MEAN, typename V>
+// FORM 1, 2: the gravity of Eq. Gravity_1, Eq. Gravity_2; 0: either, with rho_ref or
+// -(<rho> - rho_ref) in the place of dmean
+template <int FORM, typename V>
 __device__ __forceinline__ Velocity<V> unit_velocity(V dr, V jx, V jy, V psi, V Sx, V Sy, V dmean, const UnitT<V>& k,
                                                      V& Fx, V& Fy) {
-  const V half = cst<V>(0.5);
   const V rho = k.p.rho_ref + dr;
-  const V base = MEAN ? (dr - dmean) : rho;
+  const V base = FORM == 2 ? dr - dmean : (FORM == 1 ? rho : dr + dmean);
   const V t = k.p.negG * psi;
   Fx = fmadd(t, Sx, base * k.p.gx);
   Fy = fmadd(t, Sy, base * k.p.gy);
   const V inv = unit_rcp(rho);
-  return {rho, fmadd(half, Fx, jx) * inv, fmadd(half, Fy, jy) * inv};  // Eq. Momentum
+  return {rho, fma2(0.5, Fx, jx) * inv, fma2(0.5, Fy, jy) * inv};  // Eq. Momentum
 }
-template <bool MEAN, typename V>
+// f* = M^-1 m* from drho, j*, A/36, p_xx* and 2 p_xy*
+template <typename V>
+__device__ __forceinline__ void unit_back(V dr, V jx, V jy, V A36, V pxx, V pq, V (&o)[9]) {
+  o[0] = fmadd(cst<V>(-8.0), A36, cst<V>(4.0 / 9.0) * dr);
+  const V ba = fmadd(cst<V>(1.0 / 9.0), dr, A36), bd = fmadd(cst<V>(1.0 / 36.0), dr, A36);
+  V tp, tm, up, um;
+  plus_minus(0.25, pxx, ba, tp, tm);
+  plus_minus(1.0 / 3.0, jx, tp, o[1], o[3]);
+  plus_minus(1.0 / 3.0, jy, tm, o[2], o[4]);
+  plus_minus(0.125, pq, bd, up, um);
+  plus_minus(1.0 / 12.0, jx + jy, up, o[5], o[7]);
+  plus_minus(1.0 / 12.0, jy - jx, um, o[6], o[8]);
+}
+// double-float: products only by 1/9 and 1/3, the other factors are powers of two
+__device__ __forceinline__ void unit_back(dd dr, dd jx, dd jy, dd A36, dd pxx, dd pq, dd (&o)[9]) {
+  const dd d9 = cst<dd>(1.0 / 9.0) * dr;
+  o[0] = scale2(4.0, d9) - scale2(8.0, A36);
+  const dd ba = d9 + A36, bd = scale2(0.25, d9) + A36;
+  const dd q = scale2(0.25, pxx), r = scale2(0.125, pq);
+  const dd tp = ba + q, tm = ba - q, up = bd + r, um = bd - r;
+  const dd x3 = cst<dd>(1.0 / 3.0) * jx, y3 = cst<dd>(1.0 / 3.0) * jy;
+  o[1] = tp + x3;
+  o[3] = tp - x3;
+  o[2] = tm + y3;
+  o[4] = tm - y3;
+  const dd s = scale2(0.25, x3 + y3), t = scale2(0.25, y3 - x3);
+  o[5] = up + s;
+  o[7] = up - s;
+  o[6] = um + t;
+  o[8] = um - t;
+}
+
+template <int FORM, typename V>
 __device__ __forceinline__ Velocity<V> unit_collide(V dr, V jx, V jy, V psi, V Sx, V Sy, V dmean, const UnitT<V>& k,
                                                     V (&o)[9]) {
   V Fx, Fy;
-  const Velocity<V> u = unit_velocity<MEAN>(dr, jx, jy, psi, Sx, Sy, dmean, k, Fx, Fy);
+  const Velocity<V> u = unit_velocity<FORM>(dr, jx, jy, psi, Sx, Sy, dmean, k, Fx, Fy);
   const V jsx = jx + Fx, jsy = jy + Fy;                       // j*
-  const V hx = fmadd(cst<V>(0.5), Fx, jsx), hy = fmadd(cst<V>(0.5), Fy, jsy);  // rho u + F
+  const V hx = fma2(0.5, Fx, jsx), hy = fma2(0.5, Fy, jsy);   // rho u + F
   const V a = u.ux * hx, b = u.uy * hy;
   const V pq = fmadd(u.ux, hy, u.uy * hx);                    // 2 p_xy*
   const V S2 = fmadd(Sx, Sx, Sy * Sy);
   const V A36 = fmadd(cst<V>(1.0 / 12.0), a + b, k.kS * S2);  // A/36
-  const V pxx = a - b;
-  o[0] = fmadd(cst<V>(-8.0), A36, cst<V>(4.0 / 9.0) * dr);
-  const V ba = fmadd(cst<V>(1.0 / 9.0), dr, A36);
-  const V tp = fmadd(cst<V>(0.25), pxx, ba), tm = fmadd(cst<V>(-0.25), pxx, ba);
-  const V third = cst<V>(1.0 / 3.0), mthird = cst<V>(-1.0 / 3.0);
-  o[1] = fmadd(third, jsx, tp);
-  o[3] = fmadd(mthird, jsx, tp);
-  o[2] = fmadd(third, jsy, tm);
-  o[4] = fmadd(mthird, jsy, tm);
-  const V bd = fmadd(cst<V>(1.0 / 36.0), dr, A36);
-  const V up = fmadd(cst<V>(0.125), pq, bd), um = fmadd(cst<V>(-0.125), pq, bd);
-  const V sxy = jsx + jsy, dyx = jsy - jsx;
-  const V tw = cst<V>(1.0 / 12.0), mtw = cst<V>(-1.0 / 12.0);
-  o[5] = fmadd(tw, sxy, up);
-  o[7] = fmadd(mtw, sxy, up);
-  o[6] = fmadd(tw, dyx, um);
-  o[8] = fmadd(mtw, dyx, um);
+  unit_back(dr, jsx, jsy, A36, a - b, pq, o);
   return u;
 }
 
@@ -146,7 +211,9 @@ template <typename V>
 __device__ __forceinline__ void unit_zou_he(V K, bool bottom, V dmean, const UnitT<V>& k, V& dr, V& jx, V& jy) {
   const V sg = (bottom ? cst<V>(0.5) : cst<V>(-0.5)) * k.p.gy;
   const V num = (k.p.form == 2) ? fmadd(sg, dmean, K) : K - sg * k.p.rho_ref;
-  dr = fast_div(num, cst<V>(1.0) + sg);
+  // num/(1 + s) = num - num s/(1 + s): s is small, so its rounding does not move the density the
+  // same way at every step, as a rounded factor 1/(1 + s) would
+  dr = fmadd(cst<V>(-1.0) * fast_div(sg, cst<V>(1.0) + sg), num, num);
   const V base = (k.p.form == 2) ? (dr - dmean) : (k.p.rho_ref + dr);
   const V mh = cst<V>(-0.5);
   jx = mh * (base * k.p.gx);

@@ -31,6 +31,7 @@
 // register renaming; rows are loaded three ahead.
 #include "lbm_dd.cuh"
 #include "lbm_internal.h"
+#include "lbm_lane.cuh"
 #include "lbm_ptx.cuh"
 #include "lbm_unit.cuh"
 
@@ -55,10 +56,6 @@ template <>
 struct LaneOf<double> {
   using V = double;
   static constexpr int N = 2;
-};
-template <typename V, int N>
-struct Lane {
-  V v[N];
 };
 template <typename T>
 using LaneT = Lane<typename LaneOf<T>::V, LaneOf<T>::N>;
@@ -94,80 +91,13 @@ __device__ __forceinline__ void store_doubles(double* p, const Lane<f2, N>& q) {
 }
 
 // value at x - 1 / x + 1 of every column; the segment's edge lanes get their own value there
-template <int N>
-__device__ __forceinline__ Lane<f2, N> from_left(const Lane<f2, N>& q, int seg) {
-  Lane<f2, N> o;
-  o.v[0] = make_f2(__shfl_up_sync(0xffffffffu, hi(q.v[N - 1]), 1, seg), lo(q.v[0]));
-#pragma unroll
-  for (int j = 1; j < N; ++j) o.v[j] = make_f2(hi(q.v[j - 1]), lo(q.v[j]));
-  return o;
-}
-template <int N>
-__device__ __forceinline__ Lane<f2, N> from_right(const Lane<f2, N>& q, int seg) {
-  Lane<f2, N> o;
-  o.v[N - 1] = make_f2(hi(q.v[N - 1]), __shfl_down_sync(0xffffffffu, lo(q.v[0]), 1, seg));
-#pragma unroll
-  for (int j = 0; j + 1 < N; ++j) o.v[j] = make_f2(hi(q.v[j]), lo(q.v[j + 1]));
-  return o;
-}
-template <int N>
-__device__ __forceinline__ Lane<double, N> from_left(const Lane<double, N>& q, int seg) {
-  Lane<double, N> o;
-  o.v[0] = __shfl_up_sync(0xffffffffu, q.v[N - 1], 1, seg);
-#pragma unroll
-  for (int j = 1; j < N; ++j) o.v[j] = q.v[j - 1];
-  return o;
-}
-template <int N>
-__device__ __forceinline__ Lane<double, N> from_right(const Lane<double, N>& q, int seg) {
-  Lane<double, N> o;
-  o.v[N - 1] = __shfl_down_sync(0xffffffffu, q.v[0], 1, seg);
-#pragma unroll
-  for (int j = 0; j + 1 < N; ++j) o.v[j] = q.v[j + 1];
-  return o;
-}
-
 template <typename V, int N>
-__device__ __forceinline__ Lane<V, N> operator+(const Lane<V, N>& x, const Lane<V, N>& y) {
-  Lane<V, N> o;
-#pragma unroll
-  for (int j = 0; j < N; ++j) o.v[j] = x.v[j] + y.v[j];
-  return o;
+__device__ __forceinline__ Lane<V, N> from_left(const Lane<V, N>& q, int seg) {
+  return shift_left(q, [seg](auto v) { return __shfl_up_sync(0xffffffffu, v, 1, seg); });
 }
 template <typename V, int N>
-__device__ __forceinline__ Lane<V, N> operator-(const Lane<V, N>& x, const Lane<V, N>& y) {
-  Lane<V, N> o;
-#pragma unroll
-  for (int j = 0; j < N; ++j) o.v[j] = x.v[j] - y.v[j];
-  return o;
-}
-template <typename V, int N>
-__device__ __forceinline__ Lane<V, N> operator*(V s, const Lane<V, N>& x) {
-  Lane<V, N> o;
-#pragma unroll
-  for (int j = 0; j < N; ++j) o.v[j] = s * x.v[j];
-  return o;
-}
-template <typename V, int N>
-__device__ __forceinline__ Lane<V, N> fma_lane(V s, const Lane<V, N>& x, const Lane<V, N>& y) {
-  Lane<V, N> o;
-#pragma unroll
-  for (int j = 0; j < N; ++j) o.v[j] = fmadd(s, x.v[j], y.v[j]);
-  return o;
-}
-template <typename V, int N>
-__device__ __forceinline__ V sum_lane(const Lane<V, N>& x) {
-  V o = x.v[0];
-#pragma unroll
-  for (int j = 1; j < N; ++j) o = o + x.v[j];
-  return o;
-}
-template <typename V, int N>
-__device__ __forceinline__ Lane<V, N> splat_lane(V s) {
-  Lane<V, N> o;
-#pragma unroll
-  for (int j = 0; j < N; ++j) o.v[j] = s;
-  return o;
+__device__ __forceinline__ Lane<V, N> from_right(const Lane<V, N>& q, int seg) {
+  return shift_right(q, [seg](auto v) { return __shfl_down_sync(0xffffffffu, v, 1, seg); });
 }
 
 // sum over the warp of the lanes' mass partials, in every lane: the FP32 accumulators' two-sum
@@ -313,7 +243,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? kWalkThreadsF : kWalkThreadsD
       for (int j = 0; j < N; ++j) {
         V Fx, Fy;
         const Velocity<V> u =
-            unit_velocity<MEAN>(dr1.v[j], jx1.v[j], jy1.v[j], psi1.v[j], Sx.v[j], Sy.v[j], dmean, k, Fx, Fy);
+            unit_velocity<MEAN ? 2 : 1>(dr1.v[j], jx1.v[j], jy1.v[j], psi1.v[j], Sx.v[j], Sy.v[j], dmean, k, Fx, Fy);
         rho.v[j] = u.rho;
         ux.v[j] = u.ux;
         uy.v[j] = u.uy;
@@ -330,7 +260,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? kWalkThreadsF : kWalkThreadsD
       for (int j = 0; j < N; ++j) {
         V o[9];
         const Velocity<V> u =
-            unit_collide<MEAN>(dr1.v[j], jx1.v[j], jy1.v[j], psi1.v[j], Sx.v[j], Sy.v[j], dmean, k, o);
+            unit_collide<MEAN ? 2 : 1>(dr1.v[j], jx1.v[j], jy1.v[j], psi1.v[j], Sx.v[j], Sy.v[j], dmean, k, o);
 #pragma unroll
         for (int i = 0; i < 9; ++i) f[i].v[j] = o[i];
         rho.v[j] = u.rho;
