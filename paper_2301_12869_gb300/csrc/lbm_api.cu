@@ -7,6 +7,7 @@
 // used to build initial conditions and the interface level of
 // LBM_REDUCE_INTERFACE_Y. All arithmetic of the time step runs in the kernels.
 #include "lbm.h"
+#include "lbm_column.h"
 #include "lbm_internal.h"
 #include "lbm_ptx.cuh"
 
@@ -145,6 +146,8 @@ struct lbm_handle {
   lbm::WalkTiling walk{};
   bool pop = true, mom = false;
   int mcur = 0;
+  bool parts_ok = true;  // parts[pcur] are the partial sums of f[cur] (when not mom)
+  lbm::ColumnPlan column{};  // a small lattice is stepped on chip (ok: it fits)
   int since_io = 0;      // population steps since the populations were last set or read
   void* m(int b) const { return static_cast<char*>(f[1 - cur]) + size_t(3 * b) * N * s; }
   double* mean(int b) const { return red + 4 + b; }  // Zou-He: <rho> - rho_ref for the collision of m(b)
@@ -333,6 +336,49 @@ bool walk_usable(const lbm_handle* h) {
 }
 bool walk_eligible(const lbm_handle* h) { return h->tiling.variant == 0 && walk_usable(h); }
 
+// Lattices small enough for one cluster are stepped on chip, any number of steps a launch: FP32
+// up to 2^15 nodes 128 wide (64 x 128: 2.6 us a step, 4.6 walked, 6.7 on populations), FP64 up to
+// 2^12 nodes 32 wide (4 x 200: 4.7 us a step against 13.6 on populations: a node a lane is 99 FP64
+// instructions of 61 clocks, 3.1 us; beyond, the FP64 pipes of eight SMs take longer than all).
+bool column_fits(const lbm_params& p) {
+  const long long n = (long long)p.nx * p.ny;
+  return !p.thermal && n <= (p.precision == LBM_FP32 ? 1 << 15 : 1 << 12);
+}
+bool column_usable(const lbm_handle* h) { return h->column.ok && lbm::unit_relaxation(h->phys); }
+
+// nsteps steps of the populations f in place
+cudaError_t column_launch(lbm_handle* h, void* f, int64_t nsteps) {
+  lbm::ColumnArgs a{};
+  a.one = lbm::BatchCol{h->p.ny, h->p.gravity_form, 0, h->phys.RT, h->p.gx, h->p.gy, h->phys.rho_ref};
+  a.ncols = 1;
+  a.nx = h->p.nx;
+  a.f = f;
+  a.a = h->p.a;
+  a.b = h->p.b;
+  a.G = h->p.G;
+  a.sig_e = h->phys.sig_e;
+  a.status = h->status;
+  a.zh = h->p.wall == LBM_WALL_ZOU_HE;
+  cudaError_t e = cudaSuccess;
+  constexpr int64_t kMost = 1 << 20;  // steps a launch: seconds, not hours
+  for (int64_t done = 0; done < nsteps && e == cudaSuccess; done += kMost) {
+    a.run_one = lbm::RunParams{-1.0, (long long)std::min(kMost, nsteps - done), 0, 0, 0, nullptr, 0};
+    e = lbm::launch_columns(h->p.precision, h->column, false, 1, a, h->stream);
+  }
+  return e;
+}
+
+// a stream capture in progress: what is launched runs at every replay, so the form of the state
+// must not change with it
+bool capturing(const lbm_handle* h) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
 lbm::WalkIO walk_io(lbm_handle* h, int b) {  // reading m(b)
   lbm::WalkIO io{};
   io.min = h->m(b);
@@ -343,9 +389,20 @@ lbm::WalkIO walk_io(lbm_handle* h, int b) {  // reading m(b)
   return io;
 }
 
+// Fresh FP64 partials of the stored state into parts[pcur].
+int refresh_partials(lbm_handle* h) {
+  LBM_CUDA(h, lbm::launch_partials(h->p.precision, h->f[h->cur], h->p.nx, h->p.ny, h->parts[h->pcur], h->P, h->stream));
+  h->npart = h->P;
+  h->parts_ok = true;
+  return LBM_OK;
+}
+
+int ensure_partials(lbm_handle* h) { return h->parts_ok ? LBM_OK : refresh_partials(h); }
+
 // m(0) = the moments of the populations f[cur]
 int form_moments(lbm_handle* h) {
   if (h->mom) return LBM_OK;
+  if (int rc = ensure_partials(h)) return rc;
   lbm::WalkIO io{};
   io.fin = h->f[h->cur];
   io.mout = h->m(0);
@@ -369,14 +426,7 @@ int form_populations(lbm_handle* h) {
   io.fout = h->f[h->cur];
   io.Tfield = h->Tnext;  // the temperature that step used
   LBM_CUDA(h, lbm::launch_walk(h->p.precision, lbm::WALK_POPULATIONS, h->walk, h->phys, io, h->stream));
-  h->pop = true;
-  return LBM_OK;
-}
-
-// Fresh FP64 partials of the stored state into parts[pcur].
-int refresh_partials(lbm_handle* h) {
-  LBM_CUDA(h, lbm::launch_partials(h->p.precision, h->f[h->cur], h->p.nx, h->p.ny, h->parts[h->pcur], h->P, h->stream));
-  h->npart = h->P;
+  h->pop = !capturing(h);  // a captured launch has not run: the moments stay the state
   return LBM_OK;
 }
 
@@ -453,6 +503,7 @@ int run_moments(lbm_handle* h, double* rho, double* ux, double* uy) {
     LBM_CUDA(h, lbm::launch_walk(h->p.precision, lbm::WALK_MOMENTS, h->walk, h->phys, io, h->stream));
     return LBM_OK;
   }
+  if (int rc = ensure_partials(h)) return rc;
   lbm::StepIO io{};
   io.Tfield = h->Tf;
   io.fin = h->f[h->cur];
@@ -588,6 +639,10 @@ int lbm_init(const lbm_params* p, const double* rho0, int rho0_where, void* stre
   h->P = h->tiling.nbands * h->tiling.nstrips;
   h->Pcap = max_partials(*p, h->nsm, h->err);
   if (h->Pcap < 0) return fail(LBM_EINVAL);
+  if (column_fits(*p)) {
+    h->column = lbm::plan_columns(p->precision, p->nx, p->ny, p->ny, 8, p->precision == LBM_FP32 ? 0 : 64);
+    if (h->column.ok) h->column.ok = lbm::column_clusters(p->precision, h->column, false) > 0;
+  }
   lbm::plan_walk(p->precision, p->nx, p->ny, p->wall == LBM_WALL_ZOU_HE, h->nsm, h->Pcap, &h->walk);
   const Layout L = layout_for(*p, h->Pcap);
   if (p->workspace) {
@@ -668,8 +723,18 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
   lbm::TraceRange trace("lbm_step");
   if (!h) { set_err(g_err, "handle is NULL"); return LBM_EINVAL; }
   if (nsteps < 0) { set_err(h->err, "nsteps must be >= 0"); return LBM_EINVAL; }
-  if (walk_eligible(h) && (h->mom || nsteps + h->since_io >= kWalkSteps)) return walk_steps(h, nsteps);
+  const bool block = nsteps + h->since_io >= kWalkSteps;  // not a single step between reads
+  if (block && h->tiling.variant == 0 && column_usable(h)) {
+    if (int rc = leave_moments(h)) return rc;
+    if (nsteps > 0) h->parts_ok = false;
+    h->since_io = kWalkSteps;
+    LBM_CUDA(h, column_launch(h, h->f[h->cur], nsteps));
+    h->steps += nsteps;
+    return LBM_OK;
+  }
+  if (walk_eligible(h) && (h->mom || (block && !capturing(h)))) return walk_steps(h, nsteps);
   if (int rc = leave_moments(h)) return rc;
+  if (int rc = ensure_partials(h)) return rc;
   h->since_io = int(std::min<int64_t>(h->since_io + nsteps, kWalkSteps));
   lbm::StepIO io{};
   io.status = h->status;
@@ -902,6 +967,7 @@ int lbm_autotune(lbm_handle* h, int steps, int* variant, double* ms) {
   if (!h) { set_err(g_err, "handle is NULL"); return LBM_EINVAL; }
   if (steps < 1) { set_err(h->err, "steps must be >= 1"); return LBM_EINVAL; }
   if (int rc0 = leave_moments(h)) return rc0;
+  if (int rc0 = ensure_partials(h)) return rc0;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   LBM_CUDA(h, cudaEventCreate(&e0));
   cudaError_t ce = cudaEventCreate(&e1);
@@ -923,12 +989,18 @@ int lbm_autotune(lbm_handle* h, int steps, int* variant, double* ms) {
   for (int v = 0; v < lbm::step_num_variants(h->p.precision) && rc == LBM_OK; ++v) {
     lbm::StepTiling t;
     if (plan_tiling(h->p, h->nsm, &t, h->err, v)) continue;
-    // variant 0 is the step on moments where that is used: timed on moments formed in the
-    // spare buffer
-    const bool walk = v == 0 && walk_usable(h);
+    // variant 0 is the step on chip or on moments where that is used: timed on a copy of the
+    // state, or on its moments, in the spare buffer
+    const bool column = v == 0 && column_usable(h);
+    const bool walk = v == 0 && !column && walk_usable(h);
+    if (column) LBM_CUDA(h, cudaMemcpyAsync(h->f[1 - h->cur], h->f[h->cur], 9 * h->N * h->s, cudaMemcpyDeviceToDevice, h->stream));
     if (walk && (rc = form_moments(h))) break;
     cudaError_t e = cudaSuccess;
     auto launch = [&](int n) {
+      if (column) {
+        if (e == cudaSuccess) e = column_launch(h, h->f[1 - h->cur], n);
+        return;
+      }
       for (int k = 0; k < n && e == cudaSuccess && rc == LBM_OK; ++k) {
         if (walk)
           rc = walk_launch(h);

@@ -46,9 +46,10 @@ void fill_config(const ColumnPlan& p, int clusters, cudaStream_t stream, cudaLau
 
 }  // namespace
 
-ColumnPlan plan_columns(int precision, int nx, int ny, int min_ny, int cluster_goal) {
+ColumnPlan plan_columns(int precision, int nx, int ny, int min_ny, int cluster_goal, int min_items) {
   ColumnPlan p;
-  const Shape s = shape_of(precision);
+  Shape s = shape_of(precision);
+  if (min_items > 0) s.min_items = min_items;
   const int m = nx / s.Q;  // items of a row
   if (nx % s.Q || m < 1 || m > 32) return p;
   while ((1 << p.row_log2) < m) ++p.row_log2;

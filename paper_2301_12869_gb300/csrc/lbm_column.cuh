@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(ItemOf<T>::max_threads, sizeof(T) == 4 && R > 
 
     // ---- M_0: the moments of the stored populations, pulled; FP32 columns that are checked in
     // their first step also hold what FP32 does not of the density
-    const bool low_first = LOW && K <= 2;
+    const bool low_first = LOW && K == 2;
     L dr[R], jx[R], jy[R], dl[R], Kq[R];
     double kx[LOW ? R * Q : 1];
     double mass0 = 0.0;
@@ -491,12 +491,12 @@ __global__ void __launch_bounds__(ItemOf<T>::max_threads, sizeof(T) == 4 && R > 
     long long it = 0;
     const long long iters = run.max_steps;
     bool last = false;
-    int until = K;  // steps to the end of the check interval, this one included
+    int until = K >= 2 ? K : 0;  // steps to the end of the check interval, this one included (0: no checks)
     while (it < iters) {
       last = it + 1 == iters;
       const bool save = until == 2, chk = until == 1;
       const bool low_next = LOW && (until == 3 || until == 2 || (until == 1 && K == 2));
-      until = until == 1 ? K : until - 1;
+      if (until) until = until == 1 ? K : until - 1;
       if (save) {
 #pragma unroll
         for (int q = 0; q < R; ++q)

@@ -59,8 +59,9 @@ struct ColumnPlan {
 };
 
 // the launch of columns nx wide and up to ny rows tall (at least min_ny); `cluster_goal`: as many
-// CTAs a column as are useful and allowed (a power of two). precision: LBM_FP32 / FP64 / DOUBLE_FLOAT
-ColumnPlan plan_columns(int precision, int nx, int ny, int min_ny, int cluster_goal);
+// CTAs a column as are useful and allowed (a power of two); min_items: items (threads) a CTA keeps
+// when a column is split, 0: what pays when other columns wait. precision: LBM_FP32 / FP64 / DOUBLE_FLOAT
+ColumnPlan plan_columns(int precision, int nx, int ny, int min_ny, int cluster_goal, int min_items = 0);
 // resident clusters of a plan on the current device (0: it cannot run)
 int column_clusters(int precision, const ColumnPlan& p, bool acc);
 cudaError_t launch_columns(int precision, const ColumnPlan& p, bool acc, int clusters, const ColumnArgs& args,
