@@ -6,8 +6,8 @@
 // Arithmetic: bfloat16 inputs, weights and activations as matrix operands, FP32
 // accumulation, FP32 biases, output layer, loss and Adam (FP32 master weights).
 //
-// Every matrix product runs on the tcgen05 tensor cores through one GEMM kernel,
-// C[M x N] = A[M x K] B[N x K]^T with A and B bfloat16, K contiguous:
+// Every matrix product runs on the tcgen05 tensor cores. The bare product (lbm_mlp_gemm) is one
+// GEMM kernel, C[M x N] = A[M x K] B[N x K]^T with A and B bfloat16, K contiguous:
 //  * a CTA (4 warps) owns a 128 x 128 output tile whose FP32 accumulator lives in 128
 //    TMEM columns; K is consumed in chunks of 64 through kStages shared-memory stages;
 //  * one thread (the producer) fills a stage with two TMA tile copies: a 2-D tensor map
@@ -21,15 +21,15 @@
 //    refilling the stage, and after the last chunk to the `done` mbarrier;
 //  * the epilogue reads the accumulator with tcgen05.ld (warp w: rows 32w..32w+31, one row
 //    per lane), turns each 32 x 32 piece around in shared memory so that the lanes run
-//    along a row of C, and applies a fused operation with coalesced accesses: store,
-//    split-K atomic add, bias + SiLU (forward), or the SiLU derivative (backward) with the
-//    bias gradient as a column sum; transposed bfloat16 copies go out with the lanes
-//    along the rows again.
+//    along a row of C, and stores or adds (split K) it with coalesced accesses.
+// The network itself takes two fused kernels: mlp_forward_kernel (inference) and
+// mlp_train_kernel (a training step's forward and backward pass).
 // Waits are bounded (clock64); a timeout sets the status word and the CTA still waits
 // (bounded) for its MMAs and frees its TMEM before returning.
 #include "lbm.h"
 #include "lbm_internal.h"
 #include "lbm_ptx.cuh"
+#include "lbm_vec.cuh"
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -74,7 +74,7 @@ constexpr int GEMM_SMEM = 2 * kStages * TILE_BYTES + 1024 + 128;  // stages, ali
 // 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4 at bits 24-28
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(BN >> 3) << 17) | (uint32_t(BM >> 4) << 24);
 
-enum Epi : int { EPI_STORE = 0, EPI_ATOMIC = 1, EPI_FWD = 2, EPI_BWD = 3 };
+enum Epi : int { EPI_STORE = 0, EPI_ATOMIC = 1 };
 
 struct GemmArgs {
   const bf16* A;
@@ -84,14 +84,6 @@ struct GemmArgs {
   int M, N, K, k_split;  // k_split: K range per blockIdx.z (multiple of BK)
   float* C;              // EPI_STORE / EPI_ATOMIC: C[m * ldc + n]
   int ldc;
-  const float* bias;     // EPI_FWD: z = acc + bias[n]
-  float* Z;              // EPI_FWD: z stored; EPI_BWD: z read (SiLU derivative)
-  int ldz;
-  bf16* H;               // EPI_FWD: silu(z); EPI_BWD: dz = acc silu'(z)  ([m][n], may be NULL)
-  int ldh;
-  bf16* HT;              // the same values transposed ([n][m], may be NULL)
-  int ldht;
-  float* colsum;         // EPI_BWD: colsum[n] += sum over m of dz (may be NULL)
   int* status;
 };
 
@@ -117,17 +109,6 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(lbm::smem_u32(bar)), "r"(bytes)
                : "memory");
-}
-
-__device__ __forceinline__ float silu_f(float z) { return z / (1.0f + expf(-z)); }
-__device__ __forceinline__ float dsilu_f(float z) {
-  const float s = 1.0f / (1.0f + expf(-z));
-  return s * (1.0f + z * (1.0f - s));
-}
-__device__ __forceinline__ float warp_sum_f(float v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
 }
 
 template <int EPI>
@@ -220,7 +201,6 @@ __global__ void __launch_bounds__(GT, 1)
     // t[r][c] holds row 32 warp + r, column nb + c
     float* t = reinterpret_cast<float*>(smem) + warp * (32 * 33);
     const int mw = m0 + 32 * warp;
-    float csum = 0.0f;  // EPI_BWD: this lane's column sum over the warp's rows
 #pragma unroll 1
     for (int cc = 0; cc < BN / 32; ++cc) {
       float v[32];
@@ -230,7 +210,6 @@ __global__ void __launch_bounds__(GT, 1)
 #pragma unroll
       for (int i = 0; i < 32; ++i) t[lane * 33 + i] = v[i];
       __syncwarp();
-      if constexpr (EPI == EPI_BWD) csum = 0.0f;
 #pragma unroll 4
       for (int r = 0; r < 32; ++r) {
         const int m = mw + r;
@@ -238,33 +217,8 @@ __global__ void __launch_bounds__(GT, 1)
         const float x = t[r * 33 + lane];
         if constexpr (EPI == EPI_STORE) {
           if (in) g.C[size_t(m) * g.ldc + n] = x;
-        } else if constexpr (EPI == EPI_ATOMIC) {
+        } else {
           if (in) atomicAdd(g.C + size_t(m) * g.ldc + n, x);
-        } else if constexpr (EPI == EPI_FWD) {
-          if (in) {
-            const float z = x + g.bias[n];
-            g.Z[size_t(m) * g.ldz + n] = z;
-            const bf16 h = __float2bfloat16_rn(silu_f(z));
-            if (g.H) g.H[size_t(m) * g.ldh + n] = h;
-            t[r * 33 + lane] = __bfloat162float(h);
-          }
-        } else {  // EPI_BWD
-          const float dz = in ? x * dsilu_f(g.Z[size_t(m) * g.ldz + n]) : 0.0f;
-          const bf16 d = __float2bfloat16_rn(dz);
-          if (in && g.H) g.H[size_t(m) * g.ldh + n] = d;
-          t[r * 33 + lane] = __bfloat162float(d);
-          csum += dz;
-        }
-      }
-      if constexpr (EPI == EPI_FWD || EPI == EPI_BWD) {
-        if (g.colsum && n < g.N) atomicAdd(g.colsum + n, csum);
-        // the transposed copy, lanes along rows again: HT[n][m] for consecutive m
-        if (g.HT) {
-          __syncwarp();
-          const int m = mw + lane;
-#pragma unroll 4
-          for (int i = 0; i < 32; ++i)
-            if (m < g.M && nb + i < g.N) g.HT[size_t(nb + i) * g.ldht + m] = __float2bfloat16_rn(t[lane * 33 + i]);
         }
       }
       __syncwarp();
@@ -459,105 +413,345 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t counter, uint64_t seed) 
   return z ^ (z >> 31);
 }
 
-// network inputs of Bc rows: rows < count take sample first + i (or a SplitMix64 draw when
-// random), the rest are zero; X [Bc][16] and XT [16][Bc] bfloat16, targets FP32
-__global__ void gather_kernel(const float* __restrict__ feat, const float* __restrict__ tgt, long long n,
-                              long long first, int count, int random, unsigned long long seed, long long step,
-                              int Bc, bf16* __restrict__ X, bf16* __restrict__ XT, float* __restrict__ tout) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= Bc) return;
-  float x[KIN];
-#pragma unroll
-  for (int j = 0; j < KIN; ++j) x[j] = 0.0f;
-  float t = 0.0f;
-  if (i < count) {
-    const long long idx =
-        random ? (long long)(splitmix64((unsigned long long)step * (unsigned long long)count + i, seed) % (unsigned long long)n)
-               : first + i;
-#pragma unroll
-    for (int j = 0; j < LBM_MLP_INPUTS; ++j) x[j] = (feat[idx * LBM_MLP_INPUTS + j] - kCenter[j]) / kScale[j];
-    if (tgt) t = tgt[idx];
-  }
-#pragma unroll
-  for (int j = 0; j < KIN; ++j) {
-    const bf16 b = __float2bfloat16_rn(x[j]);
-    X[size_t(i) * KIN + j] = b;
-    XT[size_t(j) * Bc + i] = b;
-  }
-  if (tout) tout[i] = t;
+// ------------------------------------------------------------------ fused training pass
+// One training step's forward and backward pass over 128-row tiles, with the gradients of every
+// parameter: what took eleven launches (gather, six GEMMs with their operands and transposes in
+// global memory, a head of one row a thread) is one. A CTA of 16 warps holds the three weight
+// matrices (TMA) and a tile's operands in shared memory, and all accumulators in TMEM: the
+// layer's 128 columns, and dW3, dW2, dW1 summed over the CTA's tiles.
+//
+// Every product reads the same 128-byte-swizzled boxes (row r at 128 r bytes, 64 elements a box):
+// K-major where K runs along the rows (activations x weights of the forward pass), and
+// MN-major - the descriptor's other reading - where K is the row index: the weight gradients
+// dZ^T H sum over the tile's rows, and the backward products dZ W read W [out][in] by its rows,
+// so no transposed copy is made anywhere.
+//
+// Epilogues: warp w owns rows 32 (w % 4) .. + 31 (one a lane) and columns 32 (w / 4) .. + 31 of
+// each layer, and keeps silu'(z) of its 32 values in registers for the backward pass. The
+// gradients of b1, b2, b3 and w4 are column sums over a warp's rows (a transposing butterfly: lane
+// j ends with column j). The FP32 gradients leave the CTA once, as four-wide reductions.
+// Rounding points: bfloat16 x, W, H1, H2, dZ1..dZ3 as matrix operands; FP32 accumulation,
+// biases, output layer, loss and column sums.
+//
+// Bound by its chain of six products and epilogues, one tile a CTA (8192 rows: 64 tiles).
+constexpr int TR_THREADS = 512;
+constexpr int TR_W1 = 0;                       // W1 (K = 16, zero-filled to the box)
+constexpr int TR_W2 = TR_W1 + FF_BOX;
+constexpr int TR_W3 = TR_W2 + 2 * FF_BOX;
+constexpr int TR_X = TR_W3 + 2 * FF_BOX;       // inputs (K = 16 of a box)
+constexpr int TR_H1 = TR_X + FF_BOX;
+constexpr int TR_H2 = TR_H1 + 2 * FF_BOX;
+constexpr int TR_DZ = TR_H2 + 2 * FF_BOX;
+constexpr int TR_VEC = TR_DZ + 2 * FF_BOX;     // b1, b2, b3, w4, b4 (FP32)
+constexpr int TR_Y = TR_VEC + (4 * 128 + 4) * 4;  // [4][128] partial outputs, then [128] targets
+constexpr int TR_BAR = TR_Y + 5 * 128 * 4;
+constexpr int TR_SMEM = TR_BAR + 32 + 1024;    // + alignment slack: 203 KB
+// TMEM columns: the layer, dW3, dW2, dW1
+constexpr int TC_Z = 0, TC_W3 = 128, TC_W2 = 256, TC_W1 = 384, TC_ALL = 512;
+
+// instruction descriptor with A and / or B read MN-major (bits 15, 16), N columns
+__host__ __device__ constexpr uint32_t idesc_of(bool a_mn, bool b_mn, int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(a_mn) << 15) | (uint32_t(b_mn) << 16) |
+         (uint32_t(n >> 3) << 17) | (uint32_t(BM >> 4) << 24);
+}
+// MN-major matrix descriptor of a box pair: 64 elements along M or N a box, FF_BOX to the next
+// (leading offset), 8 rows of K in 1024 B (stride offset)
+__device__ __forceinline__ uint64_t smem_desc_mn(const void* p) {
+  const uint32_t a = lbm::smem_u32(p);
+  return uint64_t((a >> 4) & 0x3FFF) | (uint64_t(FF_BOX >> 4) << 16) | (uint64_t(1024 >> 4) << 32) |
+         (uint64_t(1) << 46) | (uint64_t(2) << 61);
 }
 
-// output layer y = silu(Z3) . w4 + b4; with train: loss, dy = 2 (y - t)/count, the
-// gradients of w4, b4, b3 and dZ3 = dy w4 silu'(Z3) (bfloat16, [Bc][128] and [128][Bc])
-__global__ void __launch_bounds__(128) head_kernel(const float* __restrict__ Z3, const float* __restrict__ P,
-                                                   const float* __restrict__ tgt, int count, int Bc, int train,
-                                                   float* __restrict__ y_out, float* __restrict__ grad,
-                                                   double* __restrict__ loss, bf16* __restrict__ dZ,
-                                                   bf16* __restrict__ dZT) {
-  __shared__ float w4[W];
-  for (int j = threadIdx.x; j < W; j += blockDim.x) w4[j] = P[OFF_W4 + j];
-  __syncthreads();
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;  // Bc is a multiple of 128: every thread has a row
+// 1/x of x >= 1 to within an FP32 rounding: the hardware's reciprocal and one Newton step
+__device__ __forceinline__ float rcp_newton(float x) {
+  const float r = lbm::rcp_approx(x);
+  return fmaf(r, fmaf(-x, r, 1.0f), r);
+}
+// silu(z) and silu'(z); d: silu' = s (1 + z (1 - s))
+__device__ __forceinline__ float silu_both(float z, float& d) {
+  const float den = 1.0f + expf(-z);
+  const float s = den < 1e30f ? rcp_newton(den) : 0.0f;  // exp overflow: sigmoid 0
+  d = s * (1.0f + z * (1.0f - s));
+  return z * s;
+}
+
+// sums over the warp's lanes of 32 values each: lane j gets the sum of v[j]. Overwrites v.
+__device__ __forceinline__ float column_sums(float (&v)[32]) {
   const int lane = threadIdx.x & 31;
-  const float* z = Z3 + size_t(s) * W;
-  float y = P[OFF_B4];
-  for (int j = 0; j < W; ++j) y += silu_f(z[j]) * w4[j];
-  const bool valid = s < count;
-  if (!train) {
-    if (valid) y_out[s] = y;
-    return;
-  }
-  const float e = valid ? y - tgt[s] : 0.0f;
-  const float dy = 2.0f * e / float(count);
-  double e2 = double(e) * double(e);
 #pragma unroll
-  for (int o = 16; o; o >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, o);
-  const float sdy = warp_sum_f(dy);
-  if (lane == 0) {
-    atomicAdd(loss, e2);
-    atomicAdd(grad + OFF_B4, sdy);
-  }
-  for (int j = 0; j < W; ++j) {
-    const float zj = z[j];
-    const float dz = dy * w4[j] * dsilu_f(zj);
-    const bf16 d = __float2bfloat16_rn(dz);
-    dZ[size_t(s) * W + j] = d;
-    dZT[size_t(j) * Bc + s] = d;
-    const float a = warp_sum_f(dz), b = warp_sum_f(silu_f(zj) * dy);
-    if (lane == 0) {
-      atomicAdd(grad + OFF_B3 + j, a);
-      atomicAdd(grad + OFF_W4 + j, b);
+  for (int m = 16; m; m >>= 1) {
+    const bool up = lane & m;
+#pragma unroll
+    for (int i = 0; i < m; ++i) {
+      const float give = up ? v[i] : v[i + m], keep = up ? v[i + m] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, m);
     }
   }
+  return v[0];
 }
 
-__global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, int n, float lr, float b1, float b2, float eps, float bc1,
-                            float bc2) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+__device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
+struct TrainArgs {
+  const float* P;
+  const float* feat;
+  const float* tgt;
+  long long n;        // samples
+  int count;          // rows of this pass: samples 0 .. count - 1, or with random SplitMix64 draws
+  int random;
+  unsigned long long seed;
+  long long step;
+  float* grad;        // += the gradients of every parameter
+  double* loss;       // += the sum of squared errors
+  int* status;
+};
+
+__global__ void __launch_bounds__(TR_THREADS, 1)
+    mlp_train_kernel(const __grid_constant__ CUtensorMap mapW1, const __grid_constant__ CUtensorMap mapW2,
+                     const __grid_constant__ CUtensorMap mapW3, const TrainArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* wbar = reinterpret_cast<uint64_t*>(smem + TR_BAR);
+  uint64_t* mbar = wbar + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + 1);
+  float* vec = reinterpret_cast<float*>(smem + TR_VEC);
+  float* ypart = reinterpret_cast<float*>(smem + TR_Y);
+  float* tgt_s = ypart + 4 * 128;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int cg = warp >> 2;                    // column group
+  const int r = 32 * (warp & 3) + lane;        // row of the tile
+  const int ntiles = (a.count + 127) / 128;
+
+  if (tid == 0) {
+    lbm::mbar_init(wbar, 1);
+    lbm::mbar_init(mbar, 1);
+    lbm::fence_mbar_init();
+  }
+  if (warp == 0) {
+    lbm::tmem_alloc(tmem_slot, TC_ALL);
+    lbm::tmem_relinquish();
+  }
+  lbm::griddep_wait();  // launched as a dependent of the parameter update
+  lbm::griddep_launch_dependents();
+  for (int i = tid; i < 4 * 128 + 1; i += TR_THREADS)
+    vec[i] = a.P[i < 128 ? OFF_B1 + i : (i < 256 ? OFF_B2 + i - 128 : (i < 384 ? OFF_B3 + i - 256 : (i < 512 ? OFF_W4 + i - 384 : OFF_B4)))];
+  lbm::tc_fence_before();
+  __syncthreads();
+  lbm::tc_fence_after();
+  const uint32_t tbase = *tmem_slot;
+  const uint32_t trow = tbase + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(32 * cg);  // this warp's lanes, columns
+  if (tid == 0) {
+    mbar_expect_tx(wbar, uint32_t(5 * FF_BOX));
+    tma_load_2d(smem + TR_W1, &mapW1, 0, 0, wbar);
+    tma_load_2d(smem + TR_W2, &mapW2, 0, 0, wbar);
+    tma_load_2d(smem + TR_W2 + FF_BOX, &mapW2, BK, 0, wbar);
+    tma_load_2d(smem + TR_W3, &mapW3, 0, 0, wbar);
+    tma_load_2d(smem + TR_W3 + FF_BOX, &mapW3, BK, 0, wbar);
+  }
+  uint32_t uses = 0;  // completed phases of mbar
+  // the CTA's writes of the operands are complete: one thread issues the products, all wait for
+  // them; false on a timeout (uniform)
+  auto products = [&](auto issue) {
+    lbm::fence_proxy_async_smem();
+    lbm::tc_fence_before();
+    __syncthreads();
+    lbm::tc_fence_after();
+    if (tid == 0) {
+      issue();
+      lbm::tc_commit(mbar);
+    }
+    const bool done = lbm::mbar_wait_bounded(mbar, uses & 1u);
+    ++uses;
+    lbm::tc_fence_after();
+    return __syncthreads_and(done) != 0;
+  };
+  auto k_off = [](int j) { return (j >> 2) * FF_BOX + 32 * (j & 3); };  // K-major step of 16
+  auto forward = [&](int src, int w, int steps) {
+    return products([&] {
+      for (int j = 0; j < steps; ++j)
+        lbm::tc_mma_f16(tbase + TC_Z, smem_desc(smem + src + k_off(j)), smem_desc(smem + w + k_off(j)),
+                        idesc_of(false, false, 128), j > 0 ? 1u : 0u);
+    });
+  };
+  bool first = true;  // the CTA's first tile: the gradients' accumulators start at zero
+  // dW (+)= dZ^T H over the tile's rows, and with wsrc the layer below: dH = dZ W
+  auto backward = [&](int h, int dw, int n, int wsrc) {
+    return products([&] {
+      for (int j = 0; j < 8; ++j)
+        lbm::tc_mma_f16(tbase + dw, smem_desc_mn(smem + TR_DZ + 2048 * j), smem_desc_mn(smem + h + 2048 * j),
+                        idesc_of(true, true, n), first && j == 0 ? 0u : 1u);
+      if (wsrc >= 0)
+        for (int j = 0; j < 8; ++j)
+          lbm::tc_mma_f16(tbase + TC_Z, smem_desc(smem + TR_DZ + k_off(j)), smem_desc_mn(smem + wsrc + 2048 * j),
+                          idesc_of(false, true, 128), j > 0 ? 1u : 0u);
+    });
+  };
+  // this warp's 32 values of a row into an operand buffer
+  auto store_row = [&](int dst, const float (&v)[32]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float piece[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) piece[i] = v[8 * q + i];
+      ff_store8(smem + dst, r, 4 * cg + q, piece);
+    }
+  };
+
+  bool ok = __syncthreads_and(lbm::mbar_wait_bounded(wbar, 0u));
+  float gb1 = 0.f, gb2 = 0.f, gb3 = 0.f, gw4 = 0.f, gb4 = 0.f;  // column 32 cg + lane over this warp's rows
+  double e2 = 0.0;
+  for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x) {
+    // ---- inputs: normalised, bfloat16, K = 16 (6 used); rows beyond count are zero
+    if (tid < 128) {
+      const int i = t * 128 + tid;
+      float x[8], z8[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) x[j] = z8[j] = 0.0f;
+      float tv = 0.0f;
+      if (i < a.count) {
+        const long long idx =
+            a.random ? (long long)(splitmix64((unsigned long long)a.step * (unsigned long long)a.count + i, a.seed) %
+                                   (unsigned long long)a.n)
+                     : i;
+#pragma unroll
+        for (int j = 0; j < LBM_MLP_INPUTS; ++j) x[j] = (a.feat[idx * LBM_MLP_INPUTS + j] - kCenter[j]) / kScale[j];
+        tv = a.tgt[idx];
+      }
+      ff_store8(smem + TR_X, tid, 0, x);
+      ff_store8(smem + TR_X, tid, 1, z8);
+      tgt_s[tid] = tv;
+    }
+    float v[32], d1[32], d2[32];
+    // ---- forward
+    if (!(ok = forward(TR_X, TR_W1, 1))) break;
+    lbm::tmem_ld32(trow + TC_Z, v);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = silu_both(v[i] + vec[32 * cg + i], d1[i]);
+    store_row(TR_H1, v);
+    if (!(ok = forward(TR_H1, TR_W2, 8))) break;
+    lbm::tmem_ld32(trow + TC_Z, v);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = silu_both(v[i] + vec[128 + 32 * cg + i], d2[i]);
+    store_row(TR_H2, v);
+    if (!(ok = forward(TR_H2, TR_W3, 8))) break;
+    lbm::tmem_ld32(trow + TC_Z, v);
+    // ---- head: y = h3 . w4 + b4, the error, and dZ3 = dy w4 silu'(z3)
+    {
+      float d3[32], yp = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        v[i] = silu_both(v[i] + vec[256 + 32 * cg + i], d3[i]);
+        yp = fmaf(v[i], vec[384 + 32 * cg + i], yp);
+      }
+      ypart[128 * cg + r] = yp;
+      __syncthreads();
+      const float y = vec[512] + ((ypart[r] + ypart[128 + r]) + (ypart[256 + r] + ypart[384 + r]));
+      const float e = t * 128 + r < a.count ? y - tgt_s[r] : 0.0f;
+      const float dy = 2.0f * e / float(a.count);
+      if (cg == 0) {
+        e2 += double(e) * double(e);
+        gb4 += dy;
+      }
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] *= dy;
+      gw4 += column_sums(v);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] = dy * vec[384 + 32 * cg + i] * d3[i];
+    }
+    store_row(TR_DZ, v);
+    gb3 += column_sums(v);
+    // ---- backward
+    if (!(ok = backward(TR_H2, TC_W3, 128, TR_W3))) break;
+    lbm::tmem_ld32(trow + TC_Z, v);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] *= d2[i];
+    store_row(TR_DZ, v);
+    gb2 += column_sums(v);
+    if (!(ok = backward(TR_H1, TC_W2, 128, TR_W2))) break;
+    lbm::tmem_ld32(trow + TC_Z, v);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] *= d1[i];
+    store_row(TR_DZ, v);
+    gb1 += column_sums(v);
+    if (!(ok = backward(TR_X, TC_W1, 16, -1))) break;
+    first = false;
+  }
+  if (ok && !first) {
+    // ---- the CTA's gradients: this warp's rows are outputs r of dW, its columns inputs; CTAs start
+    // at different pieces so that they do not queue on the same addresses
+#pragma unroll 1
+    for (int m = 0; m < 2; ++m) {
+      float v[32];
+      lbm::tmem_ld32(trow + (m == 0 ? TC_W3 : TC_W2), v);
+      float* dst = a.grad + (m == 0 ? OFF_W3 : OFF_W2) + r * W + 32 * cg;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) red_add4(dst + 4 * i, v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    }
+    if (cg == 0) {  // dW1: 16 columns
+      float v[32];
+      lbm::tmem_ld32(tbase + (uint32_t(32 * (warp & 3)) << 16) + TC_W1, v);
+      float* dst = a.grad + OFF_W1 + r * KIN;
+#pragma unroll
+      for (int i = 0; i < KIN / 4; ++i) red_add4(dst + 4 * i, v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    }
+    const int j = 32 * cg + lane;
+    atomicAdd(a.grad + OFF_B1 + j, gb1);
+    atomicAdd(a.grad + OFF_B2 + j, gb2);
+    atomicAdd(a.grad + OFF_B3 + j, gb3);
+    atomicAdd(a.grad + OFF_W4 + j, gw4);
+    if (cg == 0) {
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+        gb4 += __shfl_xor_sync(0xffffffffu, gb4, o);
+      }
+      if (lane == 0) {
+        atomicAdd(a.loss, e2);
+        atomicAdd(a.grad + OFF_B4, gb4);
+      }
+    }
+  }
+  if (!ok && tid == 0) {
+    atomicOr(a.status, lbm::STATUS_TIMEOUT);
+    // the weight copies and the issued MMAs finish before the CTA goes (bounded)
+    (void)lbm::mbar_wait_bounded(wbar, 0u, kWaitCycles / 8);
+    lbm::tc_commit(mbar);
+    (void)lbm::mbar_wait_bounded(mbar, uses & 1u, kWaitCycles / 8);
+  }
+  lbm::tc_fence_before();
+  __syncthreads();
+  if (warp == 0) lbm::tmem_dealloc(tbase, TC_ALL);
+}
+
+// Adam on the FP32 master weights (lr > 0), the gradients zeroed for the next step, and the
+// bfloat16 operand copies W1 [128][16], W2, W3 [out][in]; lr = 0: the copies alone
+__global__ void adam_kernel(float* __restrict__ P, float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
+                            float lr, float b1, float b2, float eps, float bc1, float bc2, bf16* __restrict__ W1,
+                            bf16* __restrict__ W2, bf16* __restrict__ W3) {
+  lbm::griddep_wait();  // launched as a dependent of the training pass
+  lbm::griddep_launch_dependents();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= NPARAM) return;
+  float p = P[i];
+  if (lr > 0.0f) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.0f - b1) * gi;
     const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    P[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+    p -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+    P[i] = p;
+    g[i] = 0.0f;
   }
-}
-
-// bfloat16 operand copies of the master weights: W1 [128][16], W2, W3 [out][in] and the
-// transposes W2t, W3t [in][out]
-__global__ void cast_kernel(const float* __restrict__ P, bf16* __restrict__ W1, bf16* __restrict__ W2,
-                            bf16* __restrict__ W3, bf16* __restrict__ W2t, bf16* __restrict__ W3t) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < W * KIN) W1[i] = __float2bfloat16_rn(P[OFF_W1 + i]);
-  if (i < W * W) {
-    const int o = i / W, k = i % W;
-    const bf16 a = __float2bfloat16_rn(P[OFF_W2 + i]), b = __float2bfloat16_rn(P[OFF_W3 + i]);
-    W2[i] = a;
-    W3[i] = b;
-    W2t[size_t(k) * W + o] = a;
-    W3t[size_t(k) * W + o] = b;
-  }
+  const bf16 b = __float2bfloat16_rn(p);
+  if (i < OFF_B1)
+    W1[i - OFF_W1] = b;
+  else if (i >= OFF_W2 && i < OFF_B2)
+    W2[i - OFF_W2] = b;
+  else if (i >= OFF_W3 && i < OFF_B3)
+    W3[i - OFF_W3] = b;
 }
 
 struct ColFeat {
@@ -673,17 +867,18 @@ int fail(int code, const char* fmt, ...) {
 }  // namespace
 
 // ------------------------------------------------------------------ handle
+constexpr int kLossSlots = 1024;  // training steps between two reads of their losses
+
 struct lbm_mlp {
   cudaStream_t stream = nullptr;
   int Bc = 0;  // batch capacity (multiple of 128)
   void* mem = nullptr;
   float *P = nullptr, *G = nullptr, *Mo = nullptr, *Vo = nullptr;
-  bf16 *W1 = nullptr, *W2 = nullptr, *W3 = nullptr, *W2t = nullptr, *W3t = nullptr;
-  bf16 *X = nullptr, *XT = nullptr, *H1 = nullptr, *H2 = nullptr, *H1T = nullptr, *H2T = nullptr;
-  bf16 *dZa = nullptr, *dZb = nullptr, *dZTa = nullptr, *dZTb = nullptr;
-  float *Z1 = nullptr, *Z2 = nullptr, *Z3 = nullptr, *tgt = nullptr, *y = nullptr;
-  double* loss = nullptr;
+  bf16 *W1 = nullptr, *W2 = nullptr, *W3 = nullptr;
+  CUtensorMap mW1, mW2, mW3;  // of the bfloat16 weights
+  double* loss = nullptr;     // kLossSlots sums of squared errors
   int* status = nullptr;
+  int nsm = 0;
   long long adam_t = 0;
 };
 
@@ -697,11 +892,12 @@ namespace {
 
 cudaError_t gemm_prepare() {
   cudaError_t e = cudaSuccess;
-  for (const void* fn : {(const void*)gemm_kernel<EPI_STORE>, (const void*)gemm_kernel<EPI_ATOMIC>,
-                         (const void*)gemm_kernel<EPI_FWD>, (const void*)gemm_kernel<EPI_BWD>})
+  for (const void* fn : {(const void*)gemm_kernel<EPI_STORE>, (const void*)gemm_kernel<EPI_ATOMIC>})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute((const void*)mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FF_SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute((const void*)mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TR_SMEM);
   return e;
 }
 
@@ -767,81 +963,20 @@ int status_of(lbm_mlp* h) {
   return LBM_OK;
 }
 
-// forward of rows [0, Bc) of X (count valid), then the head (train: loss and all gradients)
-int run_pass(lbm_mlp* h, int count, bool train) {
-  const int Bc = h->Bc;
-  cudaStream_t s = h->stream;
-  GemmArgs a = gargs(h->X, KIN, h->W1, KIN, Bc, W, KIN, h->status);
-  a.bias = h->P + OFF_B1;
-  a.Z = h->Z1;
-  a.ldz = W;
-  a.H = h->H1;
-  a.ldh = W;
-  a.HT = train ? h->H1T : nullptr;
-  a.ldht = Bc;
-  MLP_CUDA(gemm<EPI_FWD>(a, 1, s));
-  a = gargs(h->H1, W, h->W2, W, Bc, W, W, h->status);
-  a.bias = h->P + OFF_B2;
-  a.Z = h->Z2;
-  a.ldz = W;
-  a.H = h->H2;
-  a.ldh = W;
-  a.HT = train ? h->H2T : nullptr;
-  a.ldht = Bc;
-  MLP_CUDA(gemm<EPI_FWD>(a, 1, s));
-  a = gargs(h->H2, W, h->W3, W, Bc, W, W, h->status);
-  a.bias = h->P + OFF_B3;
-  a.Z = h->Z3;
-  a.ldz = W;
-  MLP_CUDA(gemm<EPI_FWD>(a, 1, s));
-  if (train) {
-    MLP_CUDA(cudaMemsetAsync(h->G, 0, sizeof(float) * NPARAM, s));
-    MLP_CUDA(cudaMemsetAsync(h->loss, 0, sizeof(double), s));
-  }
-  head_kernel<<<Bc / 128, 128, 0, s>>>(h->Z3, h->P, h->tgt, count, Bc, train ? 1 : 0, h->y, h->G, h->loss, h->dZa,
-                                       h->dZTa);
-  MLP_CUDA(cudaGetLastError());
-  if (!train) return LBM_OK;
-  // weight gradients are sums over the batch (K = Bc): split K over CTAs, atomic epilogue
-  const int ksplit = 1024, splits = (Bc + ksplit - 1) / ksplit;
-  auto wgrad = [&](const bf16* dZT, const bf16* HTm, int N, float* C, int ldc) {
-    GemmArgs w = gargs(dZT, Bc, HTm, Bc, W, N, Bc, h->status);
-    w.k_split = ksplit;
-    w.C = C;
-    w.ldc = ldc;
-    return gemm<EPI_ATOMIC>(w, splits, s);
-  };
-  auto dgrad = [&](const bf16* dZ, const bf16* Wt, const float* Z, bf16* dZo, bf16* dZTo, float* colsum) {
-    GemmArgs d = gargs(dZ, W, Wt, W, Bc, W, W, h->status);
-    d.Z = const_cast<float*>(Z);
-    d.ldz = W;
-    d.H = dZo;
-    d.ldh = W;
-    d.HT = dZTo;
-    d.ldht = Bc;
-    d.colsum = colsum;
-    return gemm<EPI_BWD>(d, 1, s);
-  };
-  MLP_CUDA(wgrad(h->dZTa, h->H2T, W, h->G + OFF_W3, W));                          // dW3
-  MLP_CUDA(dgrad(h->dZa, h->W3t, h->Z2, h->dZb, h->dZTb, h->G + OFF_B2));           // dZ2, db2
-  MLP_CUDA(wgrad(h->dZTb, h->H1T, W, h->G + OFF_W2, W));                          // dW2
-  MLP_CUDA(dgrad(h->dZb, h->W2t, h->Z1, h->dZa, h->dZTa, h->G + OFF_B1));           // dZ1, db1
-  MLP_CUDA(wgrad(h->dZTa, h->XT, KIN, h->G + OFF_W1, KIN));                        // dW1
-  return LBM_OK;
+// gradients (added to G) and loss (added to *loss) of rows 0 .. count - 1, or of a random minibatch
+cudaError_t train_pass(lbm_mlp* h, const float* x, const float* t, long long n, int count, bool random,
+                       unsigned long long seed, long long step, double* loss) {
+  const TrainArgs a{h->P, x, t, n, count, random ? 1 : 0, seed, step, h->G, loss, h->status};
+  const int grid = std::min(h->nsm, (count + 127) / 128);
+  return lbm::launch_dependent(mlp_train_kernel, dim3(grid), dim3(TR_THREADS), TR_SMEM, h->stream, h->mW1, h->mW2,
+                               h->mW3, a);
 }
 
-int cast_weights(lbm_mlp* h) {
-  cast_kernel<<<(W * W + 255) / 256, 256, 0, h->stream>>>(h->P, h->W1, h->W2, h->W3, h->W2t, h->W3t);
-  MLP_CUDA(cudaGetLastError());
-  return LBM_OK;
-}
-
-int gather(lbm_mlp* h, const float* x, const float* t, long long n, long long first, int count, bool random,
-           unsigned long long seed, long long step) {
-  gather_kernel<<<h->Bc / 128, 128, 0, h->stream>>>(x, t, n, first, count, random ? 1 : 0, seed, step, h->Bc, h->X,
-                                                   h->XT, h->tgt);
-  MLP_CUDA(cudaGetLastError());
-  return LBM_OK;
+cudaError_t update(lbm_mlp* h, float lr) {
+  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  const float bc1 = 1.0f - std::pow(b1, float(h->adam_t)), bc2 = 1.0f - std::pow(b2, float(h->adam_t));
+  return lbm::launch_dependent(adam_kernel, dim3((NPARAM + 255) / 256), dim3(256), 0, h->stream, h->P, h->G, h->Mo,
+                               h->Vo, lr, b1, b2, eps, bc1, bc2, h->W1, h->W2, h->W3);
 }
 
 bool device_pointer(const void* p) {
@@ -896,17 +1031,17 @@ int lbm_mlp_create(const float* params, int batch_capacity, void* stream, lbm_ml
   if (!h) return fail(LBM_ENOMEM, "out of host memory");
   h->stream = static_cast<cudaStream_t>(stream);
   h->Bc = batch_capacity;
-  const size_t Bc = size_t(batch_capacity);
   size_t off = 0;
   auto take = [&](size_t bytes) { const size_t at = off; off = (off + bytes + 255) / 256 * 256; return at; };
   const size_t oP = take(4 * NPARAM), oG = take(4 * NPARAM), oM = take(4 * NPARAM), oV = take(4 * NPARAM);
-  const size_t oW1 = take(2 * W * KIN), oW2 = take(2 * W * W), oW3 = take(2 * W * W), oW2t = take(2 * W * W),
-               oW3t = take(2 * W * W);
-  const size_t oX = take(2 * Bc * KIN), oXT = take(2 * Bc * KIN);
-  const size_t oH1 = take(2 * Bc * W), oH2 = take(2 * Bc * W), oH1T = take(2 * Bc * W), oH2T = take(2 * Bc * W);
-  const size_t odZa = take(2 * Bc * W), odZb = take(2 * Bc * W), odZTa = take(2 * Bc * W), odZTb = take(2 * Bc * W);
-  const size_t oZ1 = take(4 * Bc * W), oZ2 = take(4 * Bc * W), oZ3 = take(4 * Bc * W);
-  const size_t oT = take(4 * Bc), oY = take(4 * Bc), oL = take(8), oS = take(4);
+  const size_t oW1 = take(2 * W * KIN), oW2 = take(2 * W * W), oW3 = take(2 * W * W);
+  const size_t oL = take(8 * kLossSlots), oS = take(4);
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    delete h;
+    return fail(LBM_ECUDA, "no CUDA device");
+  }
   e = cudaMalloc(&h->mem, off);
   if (e != cudaSuccess) {
     delete h;
@@ -920,26 +1055,13 @@ int lbm_mlp_create(const float* params, int batch_capacity, void* stream, lbm_ml
   h->W1 = reinterpret_cast<bf16*>(base + oW1);
   h->W2 = reinterpret_cast<bf16*>(base + oW2);
   h->W3 = reinterpret_cast<bf16*>(base + oW3);
-  h->W2t = reinterpret_cast<bf16*>(base + oW2t);
-  h->W3t = reinterpret_cast<bf16*>(base + oW3t);
-  h->X = reinterpret_cast<bf16*>(base + oX);
-  h->XT = reinterpret_cast<bf16*>(base + oXT);
-  h->H1 = reinterpret_cast<bf16*>(base + oH1);
-  h->H2 = reinterpret_cast<bf16*>(base + oH2);
-  h->H1T = reinterpret_cast<bf16*>(base + oH1T);
-  h->H2T = reinterpret_cast<bf16*>(base + oH2T);
-  h->dZa = reinterpret_cast<bf16*>(base + odZa);
-  h->dZb = reinterpret_cast<bf16*>(base + odZb);
-  h->dZTa = reinterpret_cast<bf16*>(base + odZTa);
-  h->dZTb = reinterpret_cast<bf16*>(base + odZTb);
-  h->Z1 = reinterpret_cast<float*>(base + oZ1);
-  h->Z2 = reinterpret_cast<float*>(base + oZ2);
-  h->Z3 = reinterpret_cast<float*>(base + oZ3);
-  h->tgt = reinterpret_cast<float*>(base + oT);
-  h->y = reinterpret_cast<float*>(base + oY);
   h->loss = reinterpret_cast<double*>(base + oL);
   h->status = reinterpret_cast<int*>(base + oS);
-  int rc = lbm_mlp_set_params(h, params);
+  int rc = LBM_OK;
+  if (!make_map(&h->mW1, h->W1, W, KIN, KIN) || !make_map(&h->mW2, h->W2, W, W, W) ||
+      !make_map(&h->mW3, h->W3, W, W, W))
+    rc = fail(LBM_ECUDA, "tensor maps of the weights");
+  if (!rc) rc = lbm_mlp_set_params(h, params);
   if (rc) {
     lbm_mlp_destroy(h);
     return rc;
@@ -955,8 +1077,7 @@ int lbm_mlp_set_params(lbm_mlp* h, const float* params) {
   MLP_CUDA(cudaMemsetAsync(h->Vo, 0, sizeof(float) * NPARAM, h->stream));
   MLP_CUDA(cudaMemsetAsync(h->status, 0, sizeof(int), h->stream));
   h->adam_t = 0;
-  int rc = cast_weights(h);
-  if (rc) return rc;
+  MLP_CUDA(update(h, 0.0f));  // the bfloat16 copies
   MLP_CUDA(cudaStreamSynchronize(h->stream));
   return LBM_OK;
 }
@@ -972,13 +1093,13 @@ int lbm_mlp_gradients(lbm_mlp* h, const float* x, const float* t, int n, float* 
   if (!h || !x || !t || !grads) return fail(LBM_EINVAL, "handle, x, t and grads must not be NULL");
   if (n < 1 || n > h->Bc) return fail(LBM_EINVAL, "n must be in [1, batch_capacity]");
   if (!device_pointer(x) || !device_pointer(t)) return fail(LBM_EINVAL, "x and t must be device pointers");
-  int rc = gather(h, x, t, n, 0, n, false, 0, 0);
-  if (!rc) rc = run_pass(h, n, true);
-  if (rc) return rc;
+  MLP_CUDA(cudaMemsetAsync(h->G, 0, sizeof(float) * NPARAM, h->stream));
+  MLP_CUDA(cudaMemsetAsync(h->loss, 0, sizeof(double), h->stream));
+  MLP_CUDA(train_pass(h, x, t, n, n, false, 0, 0, h->loss));
   MLP_CUDA(cudaMemcpyAsync(grads, h->G, sizeof(float) * NPARAM, cudaMemcpyDeviceToHost, h->stream));
   double l = 0.0;
   MLP_CUDA(cudaMemcpyAsync(&l, h->loss, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  rc = status_of(h);
+  const int rc = status_of(h);
   if (loss) *loss = l / n;
   return rc;
 }
@@ -989,23 +1110,20 @@ int lbm_mlp_train(lbm_mlp* h, const float* x, const float* t, long long n, int b
   if (n < 1 || batch < 1 || batch > h->Bc || iters < 0 || !(lr > 0))
     return fail(LBM_EINVAL, "need n >= 1, 1 <= batch <= batch_capacity, iters >= 0, lr > 0");
   if (!device_pointer(x) || !device_pointer(t)) return fail(LBM_EINVAL, "x and t must be device pointers");
-  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  for (int it = 0; it < iters; ++it) {
-    int rc = gather(h, x, t, n, 0, batch, true, seed, h->adam_t);
-    if (!rc) rc = run_pass(h, batch, true);
-    if (rc) return rc;
-    ++h->adam_t;
-    const float bc1 = 1.0f - std::pow(b1, float(h->adam_t)), bc2 = 1.0f - std::pow(b2, float(h->adam_t));
-    adam_kernel<<<(NPARAM + 255) / 256, 256, 0, h->stream>>>(h->P, h->G, h->Mo, h->Vo, NPARAM, lr, b1, b2, eps, bc1,
-                                                             bc2);
-    MLP_CUDA(cudaGetLastError());
-    rc = cast_weights(h);
-    if (rc) return rc;
+  MLP_CUDA(cudaMemsetAsync(h->G, 0, sizeof(float) * NPARAM, h->stream));
+  std::vector<double> sums(losses ? std::min(iters, kLossSlots) : 0);
+  for (int first = 0; first < iters; first += kLossSlots) {
+    const int block = std::min(kLossSlots, iters - first);
+    MLP_CUDA(cudaMemsetAsync(h->loss, 0, sizeof(double) * kLossSlots, h->stream));
+    for (int it = 0; it < block; ++it) {
+      MLP_CUDA(train_pass(h, x, t, n, batch, true, seed, h->adam_t, h->loss + it));
+      ++h->adam_t;
+      MLP_CUDA(update(h, lr));
+    }
     if (losses) {
-      double l = 0.0;
-      MLP_CUDA(cudaMemcpyAsync(&l, h->loss, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+      MLP_CUDA(cudaMemcpyAsync(sums.data(), h->loss, sizeof(double) * block, cudaMemcpyDeviceToHost, h->stream));
       MLP_CUDA(cudaStreamSynchronize(h->stream));
-      losses[it] = float(l / batch);
+      for (int it = 0; it < block; ++it) losses[first + it] = float(sums[it] / batch);
     }
   }
   return status_of(h);
@@ -1017,15 +1135,10 @@ int lbm_mlp_predict(lbm_mlp* h, const float* x, long long n, float* y) {
   if (!device_pointer(x) || !device_pointer(y)) return fail(LBM_EINVAL, "x and y must be device pointers");
   if (n == 0) return LBM_OK;
   // the fused forward kernel: one persistent CTA per SM at most, four 128-row tiles in flight each
-  CUtensorMap m1, m2, m3;
-  if (!make_map(&m1, h->W1, W, KIN, KIN) || !make_map(&m2, h->W2, W, W, W) || !make_map(&m3, h->W3, W, W, W))
-    return fail(LBM_ECUDA, "tensor maps of the weights");
-  int dev = 0, nsm = 0;
-  MLP_CUDA(cudaGetDevice(&dev));
-  MLP_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   const long long ntiles = (n + 127) / 128;
-  const int grid = int(std::min<long long>(nsm, (ntiles + FF_GROUPS - 1) / FF_GROUPS));
-  mlp_forward_kernel<<<grid, FF_THREADS, FF_SMEM, h->stream>>>(m1, m2, m3, h->P, x, n, y, h->status);
+  const int grid = int(std::min<long long>(h->nsm, (ntiles + FF_GROUPS - 1) / FF_GROUPS));
+  mlp_forward_kernel<<<grid, FF_THREADS, FF_SMEM, h->stream>>>(h->mW1, h->mW2, h->mW3, h->P, x, n, y,
+                                                                 h->status);
   MLP_CUDA(cudaGetLastError());
   return status_of(h);
 }
