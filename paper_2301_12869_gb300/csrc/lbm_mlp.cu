@@ -244,8 +244,8 @@ __global__ void __launch_bounds__(GT, 1)
 // third layer the output layer is a dot product with w4 in registers. Rounding points as
 // in the GEMM path: bfloat16 inputs, weights and H1, H2; FP32 accumulation, biases, H3
 // and output.
-constexpr int FF_GROUPS = 4;                         // tile pipelines per CTA
-constexpr int FF_THREADS = 128 * FF_GROUPS;           // one group = 4 warps = 128 rows
+constexpr int FF_GROUPS = 4;                         // most tile pipelines per CTA
+constexpr int FF_THREADS = 512;                      // 16 warps
 constexpr int FF_BOX = BK * 128 * 2;                 // one 64-element x 128-row swizzled box: 16 KB
 constexpr int FF_W1 = 0;                             // W1 (K = 16, zero-filled to the box)
 constexpr int FF_W2 = FF_W1 + FF_BOX;                // W2: two K boxes
@@ -270,34 +270,55 @@ __device__ __forceinline__ void ff_store8(uint8_t* base, int r, int j, const flo
                : "memory");
 }
 
-__device__ __forceinline__ float silu_fast(float z) { return __fdividef(z, 1.0f + __expf(-z)); }
+// z / (1 + exp(-z)) of a pair: the hardware's exponential and reciprocal (a few ulp)
+__device__ __forceinline__ lbm::f2 silu_fast(lbm::f2 z) {
+  const lbm::f2 t = z * lbm::cst<lbm::f2>(-1.4426950408889634);
+  float e0, e1;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(lbm::lo(t)));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(lbm::hi(t)));
+  const lbm::f2 d = lbm::cst<lbm::f2>(1.0) + lbm::make_f2(e0, e1);
+  return z * lbm::make_f2(lbm::rcp_approx(lbm::lo(d)), lbm::rcp_approx(lbm::hi(d)));
+}
+// the pair as bfloat16, the first value in the low half
+__device__ __forceinline__ uint32_t bf16_pair(lbm::f2 v) {
+  const __nv_bfloat162 b = __floats2bfloat162_rn(lbm::lo(v), lbm::hi(v));
+  return *reinterpret_cast<const uint32_t*>(&b);
+}
 
-// barrier among the 128 threads of group g (named barrier 1 + g) returning the AND of v
-__device__ __forceinline__ bool group_and(bool v, int g) {
+// barrier among the `count` threads of group g (named barrier 1 + g) returning the AND of v
+__device__ __forceinline__ bool group_and(bool v, int g, int count) {
   uint32_t r;
   asm volatile(
       "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.b32 p, %1, 0;\n\t"
-      "bar.red.and.pred q, %2, 128, p;\n\t"
+      "bar.red.and.pred q, %2, %3, p;\n\t"
       "selp.u32 %0, 1, 0, q;\n\t}"
       : "=r"(r)
-      : "r"(uint32_t(v)), "r"(1 + g)
+      : "r"(uint32_t(v)), "r"(1 + g), "r"(count)
       : "memory");
   return r != 0;
 }
 
+// G: tile pipelines of the CTA's 16 warps - four of 4 warps (a thread does a row), or one of 16 (a
+// thread does 32 columns of a row), which takes a quarter of the time for a single tile
+template <int G>
 __global__ void __launch_bounds__(FF_THREADS, 1)
     mlp_forward_kernel(const __grid_constant__ CUtensorMap mapW1, const __grid_constant__ CUtensorMap mapW2,
                        const __grid_constant__ CUtensorMap mapW3, const float* __restrict__ P,
                        const float* __restrict__ feat, long long n, float* __restrict__ y, int* status) {
+  using lbm::f2;
+  constexpr int COLS = 32 * G;          // columns a thread does of its row
+  constexpr int GT_ = FF_THREADS / G;   // threads of a group
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* wbar = reinterpret_cast<uint64_t*>(smem + FF_BAR);
   uint64_t* mbars = wbar + 1;  // one per group
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbars + FF_GROUPS);
   float* vec = reinterpret_cast<float*>(smem + FF_VEC);  // b1 [0, 128), b2, b3, w4, b4 [512]
+  float* ypart = reinterpret_cast<float*>(smem + FF_H + 2 * FF_BOX);  // G = 1: partial outputs [4][128]
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int g = warp >> 2, r = tid & 127;  // group, and this thread's row within the tile
+  const int g = tid / GT_, cg = (tid % GT_) >> 7;        // group, column group
+  const int r = 32 * (warp & 3) + (tid & 31);            // this thread's row within the tile
   const long long ntiles = (n + 127) / 128;
 
   if (tid == 0) {
@@ -308,14 +329,14 @@ __global__ void __launch_bounds__(FF_THREADS, 1)
   for (int i = tid; i < 4 * 128 + 1; i += FF_THREADS)
     vec[i] = P[i < 128 ? OFF_B1 + i : (i < 256 ? OFF_B2 + i - 128 : (i < 384 ? OFF_B3 + i - 256 : (i < 512 ? OFF_W4 + i - 384 : OFF_B4)))];
   if (warp == 0) {
-    lbm::tmem_alloc(tmem_slot, 128 * FF_GROUPS);
+    lbm::tmem_alloc(tmem_slot, 128 * G);
     lbm::tmem_relinquish();
   }
   lbm::tc_fence_before();
   __syncthreads();
   lbm::tc_fence_after();
-  const uint32_t tmem = *tmem_slot + uint32_t(128 * g) + (uint32_t(32 * (warp & 3)) << 16);  // group columns, warp lanes
   const uint32_t tmem_acc = *tmem_slot + uint32_t(128 * g);
+  const uint32_t tmem = tmem_acc + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(COLS * cg);  // warp lanes, columns
   uint8_t* sH = smem + FF_H + g * 2 * FF_BOX;
   uint64_t* mbar = &mbars[g];
   if (tid == 0) {  // the three weight matrices, once per CTA
@@ -326,16 +347,17 @@ __global__ void __launch_bounds__(FF_THREADS, 1)
     tma_load_2d(smem + FF_W3, &mapW3, 0, 0, wbar);
     tma_load_2d(smem + FF_W3 + FF_BOX, &mapW3, BK, 0, wbar);
   }
-  bool ok = __syncthreads_and(lbm::mbar_wait_bounded(wbar, 0u));
-  uint32_t uses = 0;  // completed phases of this group's mbarrier
+  bool ok = true, weights = false;  // the weights are waited for before the first product
+  uint32_t uses = 0;                // completed phases of this group's mbarrier
   // one layer: the group's A buffer is complete; one thread issues k_steps K = 16 MMAs of
   // A (sH) and B (weights) into the group's accumulator and commits them to its mbarrier
   auto mma_layer = [&](const uint8_t* sB, int k_steps) {
     lbm::fence_proxy_async_smem();  // this group's st.shared of A -> visible to the tensor cores
     lbm::tc_fence_before();
-    (void)group_and(true, g);
+    if (!weights) weights = lbm::mbar_wait_bounded(wbar, 0u);
+    if (!group_and(weights, g, GT_)) return false;
     lbm::tc_fence_after();
-    if (r == 0) {
+    if (tid % GT_ == 0) {
       for (int j = 0; j < k_steps; ++j) {
         const int off = (j >> 2) * FF_BOX + 32 * (j & 3);
         lbm::tc_mma_f16(tmem_acc, smem_desc(sH + off), smem_desc(sB + off), kIdesc, j > 0 ? 1u : 0u);
@@ -345,11 +367,12 @@ __global__ void __launch_bounds__(FF_THREADS, 1)
     const bool done = lbm::mbar_wait_bounded(mbar, uses & 1u);
     ++uses;
     lbm::tc_fence_after();
-    return group_and(done, g);
+    return group_and(done, g, GT_);
   };
-  for (long long t = FF_GROUPS * (long long)blockIdx.x + g; ok && t < ntiles; t += FF_GROUPS * (long long)gridDim.x) {
+  // tile t of the CTA's sequence goes to its group t % G: CTAs have the same number of tiles but one
+  for (long long t = blockIdx.x + (long long)gridDim.x * g; t < ntiles; t += (long long)gridDim.x * G) {
     const long long m = t * 128 + r;  // this thread's row
-    {  // normalised inputs, bfloat16, K = 16 (6 used)
+    if (cg == 0) {  // normalised inputs, bfloat16, K = 16 (6 used)
       float a[8], b[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) a[j] = b[j] = 0.0f;
@@ -360,7 +383,7 @@ __global__ void __launch_bounds__(FF_THREADS, 1)
       ff_store8(sH, r, 0, a);
       ff_store8(sH, r, 1, b);
     }
-    float out = vec[512];
+    float out = cg == 0 ? vec[512] : 0.0f;
 #pragma unroll 1
     for (int layer = 0; layer < 3; ++layer) {
       const uint8_t* sB = smem + (layer == 0 ? FF_W1 : (layer == 1 ? FF_W2 : FF_W3));
@@ -368,41 +391,57 @@ __global__ void __launch_bounds__(FF_THREADS, 1)
         ok = false;
         break;
       }
-      const float* bias = vec + 128 * layer;
+      const float* bias = vec + 128 * layer + COLS * cg;
 #pragma unroll 1
-      for (int cc = 0; cc < 4; ++cc) {  // columns 32 cc .. 32 cc + 31 of this row
+      for (int cc = 0; cc < G; ++cc) {  // 32 of the thread's columns
         float v[32];
         lbm::tmem_ld32(tmem + uint32_t(32 * cc), v);
+        f2 h[16];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = silu_fast(v[i] + bias[32 * cc + i]);
+        for (int i = 0; i < 16; ++i)
+          h[i] = silu_fast(lbm::make_f2(v[2 * i], v[2 * i + 1]) + *reinterpret_cast<const f2*>(bias + 32 * cc + 2 * i));
         if (layer < 2) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            float piece[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) piece[i] = v[8 * q + i];
-            ff_store8(sH, r, 4 * cc + q, piece);
+          for (int q = 0; q < 4; ++q) {  // 16-byte piece j of row r at piece position j ^ (r mod 8)
+            const int j = (COLS * cg) / 8 + 4 * cc + q;
+            uint8_t* dst = sH + (j >> 3) * FF_BOX + r * 128 + (((j & 7) ^ (r & 7)) << 4);
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(lbm::smem_u32(dst)),
+                         "r"(bf16_pair(h[4 * q])), "r"(bf16_pair(h[4 * q + 1])), "r"(bf16_pair(h[4 * q + 2])),
+                         "r"(bf16_pair(h[4 * q + 3]))
+                         : "memory");
           }
         } else {
+          const float* w4 = vec + 384 + COLS * cg + 32 * cc;
 #pragma unroll
-          for (int i = 0; i < 32; ++i) out = fmaf(v[i], vec[384 + 32 * cc + i], out);
+          for (int i = 0; i < 16; ++i) {
+            out = fmaf(lbm::lo(h[i]), w4[2 * i], out);
+            out = fmaf(lbm::hi(h[i]), w4[2 * i + 1], out);
+          }
         }
       }
       // every read of the accumulator is complete before the group's next MMAs overwrite it
       lbm::tc_fence_before();
     }
-    if (ok && m < n) y[m] = out;
+    if (!ok) break;
+    if constexpr (G == 1) {  // the four column groups' parts of a row's output
+      ypart[128 * cg + r] = out;
+      __syncthreads();
+      if (cg == 0 && m < n) y[m] = (out + ypart[128 + r]) + (ypart[256 + r] + ypart[384 + r]);
+    } else if (m < n) {
+      y[m] = out;
+    }
   }
-  if (!ok && r == 0) {
+  if (!ok && tid % GT_ == 0) {
     atomicOr(status, lbm::STATUS_TIMEOUT);
-    // the weight copies and this group's issued MMAs finish before the CTA goes (bounded)
-    (void)lbm::mbar_wait_bounded(wbar, 0u, kWaitCycles / 8);
+    // this group's issued MMAs finish before the CTA goes (bounded)
     lbm::tc_commit(mbar);
     (void)lbm::mbar_wait_bounded(mbar, uses & 1u, kWaitCycles / 8);
   }
+  // the weight copies land before the CTA goes (bounded), also where no tile waited for them
+  if (!weights) (void)lbm::mbar_wait_bounded(wbar, 0u, kWaitCycles / 8);
   lbm::tc_fence_before();
   __syncthreads();
-  if (warp == 0) lbm::tmem_dealloc(*tmem_slot, 128 * FF_GROUPS);
+  if (warp == 0) lbm::tmem_dealloc(*tmem_slot, 128 * G);
 }
 
 // ------------------------------------------------------------------ other kernels
@@ -895,7 +934,9 @@ cudaError_t gemm_prepare() {
   for (const void* fn : {(const void*)gemm_kernel<EPI_STORE>, (const void*)gemm_kernel<EPI_ATOMIC>})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute((const void*)mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FF_SMEM);
+    e = cudaFuncSetAttribute((const void*)mlp_forward_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, FF_SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute((const void*)mlp_forward_kernel<FF_GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, FF_SMEM);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute((const void*)mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TR_SMEM);
   return e;
@@ -1134,11 +1175,12 @@ int lbm_mlp_predict(lbm_mlp* h, const float* x, long long n, float* y) {
   if (n < 0) return fail(LBM_EINVAL, "n must be >= 0");
   if (!device_pointer(x) || !device_pointer(y)) return fail(LBM_EINVAL, "x and y must be device pointers");
   if (n == 0) return LBM_OK;
-  // the fused forward kernel: one persistent CTA per SM at most, four 128-row tiles in flight each
+  // the fused forward kernel, one persistent CTA per SM at most: all its warps on a tile while there
+  // are no more tiles than SMs, four tiles in flight beyond
   const long long ntiles = (n + 127) / 128;
-  const int grid = int(std::min<long long>(h->nsm, (ntiles + FF_GROUPS - 1) / FF_GROUPS));
-  mlp_forward_kernel<<<grid, FF_THREADS, FF_SMEM, h->stream>>>(h->mW1, h->mW2, h->mW3, h->P, x, n, y,
-                                                                 h->status);
+  const int grid = int(std::min<long long>(h->nsm, ntiles));
+  auto fn = ntiles <= h->nsm ? mlp_forward_kernel<1> : mlp_forward_kernel<FF_GROUPS>;
+  fn<<<grid, FF_THREADS, FF_SMEM, h->stream>>>(h->mW1, h->mW2, h->mW3, h->P, x, n, y, h->status);
   MLP_CUDA(cudaGetLastError());
   return status_of(h);
 }
