@@ -23,6 +23,7 @@
 #include "lbm_internal.h"
 #include "lbm_dd.cuh"
 #include "lbm_physics.cuh"
+#include "lbm_unit.cuh"
 
 #include <cuda_runtime.h>
 
@@ -87,6 +88,9 @@ __device__ lbm::PhysT<T> column_phys(const BatchArgs& a, const BatchCol& c) {
   k.h_q = lbm::from_double<T>(1.0 - 0.5 * a.s_q); k.h_nu = lbm::from_double<T>(1.0 - 0.5 * a.s_nu);
   k.sig_e = lbm::from_double<T>(a.sig_e);
   k.nsig_vs = lbm::from_double<T>(-a.sig_vs);
+  k.k2 = lbm::from_double<T>(-2.0 * a.a / a.G);
+  k.k3 = lbm::from_double<T>(-2.0 / (3.0 * a.G));
+  k.kS = lbm::from_double<T>(a.G * a.G * a.sig_e / 72.0);
   k.gx = lbm::from_double<T>(c.gx);
   k.gy = lbm::from_double<T>(c.gy);
   k.form = c.form;

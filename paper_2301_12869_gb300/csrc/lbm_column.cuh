@@ -90,9 +90,9 @@ __device__ UnitT<V> column_unit(const ColumnArgs& a, const BatchCol& c) {
   u.p.gy = real<V>(c.gy);
   u.p.form = c.form;
   u.k1 = real<V>(2.0 * c.RT / a.G);
-  u.k2 = real<V>(-2.0 * a.a / a.G);
-  u.k3 = real<V>(-2.0 / (3.0 * a.G));
-  u.kS = real<V>(a.G * a.G * a.sig_e / 72.0);
+  u.p.k2 = real<V>(-2.0 * a.a / a.G);
+  u.p.k3 = real<V>(-2.0 / (3.0 * a.G));
+  u.p.kS = real<V>(a.G * a.G * a.sig_e / 72.0);
   return u;
 }
 

@@ -571,8 +571,10 @@ __global__ void __launch_bounds__((NWC + 1) * 32, MINB)
       const V RT = TH ? k.R * make_f2(Th, Th) : k.RT;
       return lo(psi_of<V>(k.rho_ref + make_f2(rh, rh), RT, k, flag));
     };
-    // g: the pulled populations of row y, kept in registers since its psi pass
-    auto collide = [&](int y, const V (&g)[9], const PsiRow& ps, const PsiRow& pc, const PsiRow& pn) {
+    // g: what the collision needs of row y's pulled populations, kept in registers since its psi
+    // pass - with every relaxation time 1 their three moments, else all nine
+    constexpr int NG = UNIT ? 3 : 9;
+    auto collide = [&](int y, const V (&g)[NG], const PsiRow& ps, const PsiRow& pc, const PsiRow& pn) {
       const bool lo_wall = (y == tl.ylo), hi_wall = (y == tl.yhi);
       V Sx = cst<V>(0.0), Sy = cst<V>(0.0);
       if (!lo_wall && !hi_wall) {  // Eq. ShanChenForce stencil: w(1) = 1/3, w(2) = 1/12
@@ -584,7 +586,10 @@ __global__ void __launch_bounds__((NWC + 1) * 32, MINB)
         Sy = fmadd(c13, pn.c - ps.c, c112 * ((En + Wn) - (Es + Ws)));
       }
       V o[9], rho, ux, uy;
-      collide_node<V, UNIT>(g, pc.c, Sx, Sy, dmean, k, o, rho, ux, uy, flag);
+      if constexpr (UNIT)
+        collide_moments(Moments<V>{g[0], g[1], g[2]}, pc.c, Sx, Sy, dmean, k, o, rho, ux, uy, flag);
+      else
+        collide_node<V, UNIT>(g, pc.c, Sx, Sy, dmean, k, o, rho, ux, uy, flag);
       const size_t node = size_t(y) * nx + xa + (j - 1);
       if (MODE == MODE_STEP) {
         const size_t plane = size_t(ny) * nx;
@@ -606,9 +611,9 @@ __global__ void __launch_bounds__((NWC + 1) * 32, MINB)
     };
 
     bool failed = false;
-    V gp[9];  // pulled populations of walk row kk - 1
+    V gp[NG];  // of walk row kk - 1
 #pragma unroll
-    for (int i = 0; i < 9; ++i) gp[i] = cst<V>(0.0);
+    for (int i = 0; i < NG; ++i) gp[i] = cst<V>(0.0);
     // two rows per iteration: the row state rotates by renaming instead of copies (the
     // Zou-He kernels, with their wall-row code, would spill)
     constexpr int kRowUnroll = ZH ? 1 : 2;
@@ -651,7 +656,7 @@ __global__ void __launch_bounds__((NWC + 1) * 32, MINB)
       PsiRow nw;
       if (active) {
         const V RT = TH ? k.R * Tq : k.RT;
-        nw.c = psi_of<V>(k.rho_ref + sum9(g), RT, k, flag);
+        nw.c = psi_of<V>(k.rho_ref + sum9(g), RT, k, flag);  // (the sum is the moments' too)
       } else {
         nw.c = cst<V>(0.0);
       }
@@ -672,8 +677,15 @@ __global__ void __launch_bounds__((NWC + 1) * 32, MINB)
             collide(y, gp, pp, p0, pm);
         }
       }
+      if constexpr (UNIT) {
+        const Moments<V> m = moments_of(g);
+        gp[0] = m.dr;
+        gp[1] = m.jx;
+        gp[2] = m.jy;
+      } else {
 #pragma unroll
-      for (int i = 0; i < 9; ++i) gp[i] = g[i];
+        for (int i = 0; i < 9; ++i) gp[i] = g[i];
+      }
       if constexpr (TH) Tq = Tn;
     }
     if (!failed) {  // last walk row: own only at a wall, where the stencil is not needed

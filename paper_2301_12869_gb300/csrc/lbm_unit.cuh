@@ -21,8 +21,7 @@ namespace lbm {
 template <typename V>
 struct UnitT {
   PhysT<V> p;
-  V k1, k1R, k2, k3;  // psi^2 = rho (k1 num/om^3 + k2 rho + k3): 2RT/G, 2R/G, -2a/G, -2/(3G)
-  V kS;               // G^2 sigma/(tau - 1/2)/72: the sigma term's share of A/36
+  V k1, k1R;  // 2RT/G, 2R/G
 };
 
 template <typename V>
@@ -31,47 +30,14 @@ UnitT<V> to_unit(const StepPhys& s) {
   u.p = to_phys<V>(s);
   u.k1 = host_value<V>(2.0 * s.RT / s.G);
   u.k1R = host_value<V>(2.0 * s.R / s.G);
-  u.k2 = host_value<V>(-2.0 * s.a / s.G);
-  u.k3 = host_value<V>(-2.0 / (3.0 * s.G));
-  u.kS = host_value<V>(s.G * s.G * s.sig_e / 72.0);
   return u;
 }
 
-// c x for a power of two c, and c x + y: exact scalings, which cost a double-float value two
-// multiplications instead of a product; y + c x and y - c x (one product for double-float)
-template <typename V>
-__device__ __forceinline__ V scale2(double c, V x) {
-  return cst<V>(c) * x;
-}
+// powers of two scale both parts of a double-float value exactly
 __device__ __forceinline__ dd scale2(double c, dd x) { return dd{float(c) * x.hi, float(c) * x.lo}; }
-template <typename V>
-__device__ __forceinline__ V fma2(double c, V x, V y) {
-  return fmadd(cst<V>(c), x, y);
-}
 __device__ __forceinline__ dd fma2(double c, dd x, dd y) { return scale2(c, x) + y; }
-template <typename V>
-__device__ __forceinline__ void plus_minus(double c, V x, V y, V& p, V& m) {
-  p = fmadd(cst<V>(c), x, y);
-  m = fmadd(cst<V>(-c), x, y);
-}
 
-// ---- reciprocal and reciprocal square root of a positive normal value
-// FP64: the hardware's 20-bit seed and one Householder step of third order (error of the seed
-// cubed: 2^-57), 3 and 5 FP64 instructions instead of the IEEE division's and square root's
-// 9 and more - GB300 issues an FP64 instruction per SM only every 15 clocks, so the FP64
-// step's time is the count of these. Results are within about 1 ulp.
-__device__ __forceinline__ double unit_rcp(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);  // y (1 + e + e^2)
-}
-__device__ __forceinline__ double unit_rsqrt(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-(x * y), y, 1.0);
-  return fma(fma(e, 0.375, 0.5), y * e, y);  // y (1 + e/2 + 3 e^2/8)
-}
+// ---- reciprocals of FP32 pairs and of double-float values
 __device__ __forceinline__ f2 unit_rcp(f2 x) { return make_f2(rcp_approx(lo(x)), rcp_approx(hi(x))); }
 
 // double-float: an FP32 guess (refined to 2^-23), whose correction is formed in FP32 from the
@@ -92,51 +58,34 @@ __device__ __forceinline__ dd unit_rsqrt(dd x) {
   return dd_fast_two_sum(y, __fmul_rn(__fmul_rn(y, e), __fmaf_rn(0.375f, e, 0.5f)));
 }
 
-// psi of Eqs. EOS and InteractionPotential: psi^2 = rho (k1 num/D + k2 rho + k3) with
-// D = (1 - eta)^3; psi^2 < 0 or NaN, or rho <= 0, is non-physical (psi = 0 for the former).
-// FP32 pairs: an approximate reciprocal and square root, without a branch - one would cut the
-// rows of a walk apart for the instruction scheduler.
+// psi of Eqs. EOS and InteractionPotential; rho <= 0 is non-physical as well as psi^2 < 0 or NaN.
+// FP32 pairs: without a branch - one would cut the rows of a walk apart for the instruction
+// scheduler.
 __device__ __forceinline__ f2 unit_psi(f2 rho, f2 k1, f2, const UnitT<f2>& k, int& flag) {
   const f2 one = cst<f2>(1.0);
   const f2 eta = k.p.b4 * rho;
   const f2 om = one - eta;
   const f2 num = fmadd(eta, fmadd(eta, om, one), one);  // 1 + eta + eta^2 - eta^3
   const f2 q = num * unit_rcp(om * om * om);
-  const f2 p2 = rho * fmadd(k1, q, fmadd(k.k2, rho, k.k3));
+  const f2 p2 = rho * fmadd(k1, q, fmadd(k.p.k2, rho, k.p.k3));
   const float s = lo(p2), t = hi(p2);
   if (!(s >= 0.f && t >= 0.f && lo(rho) > 0.f && hi(rho) > 0.f)) flag |= STATUS_NONPHYS;
   return make_f2(sqrt_approx(fmaxf(s, 0.f)), sqrt_approx(fmaxf(t, 0.f)));
 }
-// FP64: with N = rho (k1 num + (k2 rho + k3) D), psi = sqrt(N/D) = N rsqrt(N D): one
-// reciprocal square root in place of a division and a square root. Anything but positive
-// normal N, D and rho takes the general formula.
-__device__ __forceinline__ bool normal_positive(double x) {
-  return unsigned(__double2hiint(x)) - 0x00100000u < 0x7fe00000u;
+__device__ __forceinline__ double unit_psi(double rho, double k1, double, const UnitT<double>& k, int& flag) {
+  if (nonpositive(rho)) flag |= STATUS_NONPHYS;
+  return psi_k1(rho, k1, k.p, flag);
 }
-__device__ __forceinline__ double unit_psi(double rho, double k1, double RT, const UnitT<double>& k, int& flag) {
-  const double eta = k.p.b4 * rho;
-  const double om = 1.0 - eta;
-  const double num = fma(eta, fma(eta, om, 1.0), 1.0);
-  const double D = om * om * om;
-  const double N = rho * fma(fma(k.k2, rho, k.k3), D, k1 * num);
-  double psi = N * unit_rsqrt(N * D);
-  if (!(normal_positive(N) && normal_positive(D) && normal_positive(rho))) {
-    psi = psi_of<double>(rho, RT, k.p, flag);
-    if (nonpositive(rho)) flag |= STATUS_NONPHYS;
-  }
-  return psi;
-}
-
 __device__ __forceinline__ dd unit_psi(dd rho, dd k1, dd RT, const UnitT<dd>& k, int& flag) {
   const dd one = cst<dd>(1.0);
   const dd eta = k.p.b4 * rho;
   const dd om = one - eta;
   const dd num = fmadd(eta, fmadd(eta, om, one), one);
   const dd D = om * om * om;
-  const dd N = rho * fmadd(fmadd(k.k2, rho, k.k3), D, k1 * num);
+  const dd N = rho * fmadd(fmadd(k.p.k2, rho, k.p.k3), D, k1 * num);
   if (N.hi > 0.f && D.hi > 0.f && rho.hi > 0.f) return N * unit_rsqrt(N * D);
   if (nonpositive(rho)) flag |= STATUS_NONPHYS;
-  return psi_of<dd>(rho, RT, k.p, flag);
+  return psi_k1(rho, k1, k.p, flag);
 }
 
 // the post-collision values o of a node with moments (dr, jx, jy) before the collision, the
@@ -157,30 +106,6 @@ __device__ __forceinline__ Velocity<V> unit_velocity(V dr, V jx, V jy, V psi, V 
   Fy = fmadd(t, Sy, base * k.p.gy);
   const V inv = unit_rcp(rho);
   return {rho, fma2(0.5, Fx, jx) * inv, fma2(0.5, Fy, jy) * inv};  // Eq. Momentum
-}
-// 4 drho/9. In FP32 the rounded weights 1/9 and 1/36 exceed theirs by 7.5e-9 of drho in all, at
-// every step the same way; the rest weight takes up the difference, so that the weights add to 1
-template <typename V>
-__device__ __forceinline__ V rest_share(V dr) {
-  return cst<V>(4.0 / 9.0) * dr;
-}
-__device__ __forceinline__ f2 rest_share(f2 dr) {
-  constexpr double c = 1.0 - 5.0 * double(float(1.0 / 9.0));  // 4 (1/9) + 4 (1/36) = 5 (1/9)
-  return fmadd(cst<f2>(c), dr, cst<f2>(c - double(float(c))) * dr);
-}
-
-// f* = M^-1 m* from drho, j*, A/36, p_xx* and 2 p_xy*
-template <typename V>
-__device__ __forceinline__ void unit_back(V dr, V jx, V jy, V A36, V pxx, V pq, V (&o)[9]) {
-  o[0] = fmadd(cst<V>(-8.0), A36, rest_share(dr));
-  const V ba = fmadd(cst<V>(1.0 / 9.0), dr, A36), bd = fmadd(cst<V>(1.0 / 36.0), dr, A36);
-  V tp, tm, up, um;
-  plus_minus(0.25, pxx, ba, tp, tm);
-  plus_minus(1.0 / 3.0, jx, tp, o[1], o[3]);
-  plus_minus(1.0 / 3.0, jy, tm, o[2], o[4]);
-  plus_minus(0.125, pq, bd, up, um);
-  plus_minus(1.0 / 12.0, jx + jy, up, o[5], o[7]);
-  plus_minus(1.0 / 12.0, jy - jx, um, o[6], o[8]);
 }
 // double-float: products only by 1/9 and 1/3, the other factors are powers of two
 __device__ __forceinline__ void unit_back(dd dr, dd jx, dd jy, dd A36, dd pxx, dd pq, dd (&o)[9]) {
@@ -211,7 +136,7 @@ __device__ __forceinline__ Velocity<V> unit_collide(V dr, V jx, V jy, V psi, V S
   const V a = u.ux * hx, b = u.uy * hy;
   const V pq = fmadd(u.ux, hy, u.uy * hx);                    // 2 p_xy*
   const V S2 = fmadd(Sx, Sx, Sy * Sy);
-  const V A36 = fmadd(cst<V>(1.0 / 12.0), a + b, k.kS * S2);  // A/36
+  const V A36 = fmadd(cst<V>(1.0 / 12.0), a + b, k.p.kS * S2);  // A/36
   unit_back(dr, jsx, jsy, A36, a - b, pq, o);
   return u;
 }

@@ -123,7 +123,10 @@ __device__ __forceinline__ f2 sqrt_checked(f2 x, bool& bad) {
 }
 
 // true if any component is <= 0 or NaN
-__device__ __forceinline__ bool nonpositive(double x) { return !(x > 0.0); }
+__device__ __forceinline__ bool nonpositive(double x) {
+  // a positive normal number is told by its high word: the FP64 pipe is left alone
+  return unsigned(__double2hiint(x)) - 0x00100000u >= 0x7fe00000u && !(x > 0.0);
+}
 __device__ __forceinline__ bool nonpositive(float x) { return !(x > 0.f); }
 __device__ __forceinline__ bool nonpositive(f2 x) { return !(lo(x) > 0.f) || !(hi(x) > 0.f); }
 
