@@ -393,7 +393,7 @@ lbm::WalkIO walk_io(lbm_handle* h, int b) {  // reading m(b)
 int refresh_partials(lbm_handle* h) {
   LBM_CUDA(h, lbm::launch_partials(h->p.precision, h->f[h->cur], h->p.nx, h->p.ny, h->parts[h->pcur], h->P, h->stream));
   h->npart = h->P;
-  h->parts_ok = true;
+  h->parts_ok = !capturing(h);  // captured sums have not been formed
   return LBM_OK;
 }
 
@@ -436,6 +436,7 @@ int leave_moments(lbm_handle* h) {
   int rc = form_populations(h);
   if (rc) return rc;
   h->mom = false;
+  h->pop = true;
   return refresh_partials(h);
 }
 

@@ -1,0 +1,110 @@
+"""Small lattices of a handle, stepped on chip a block at a time, against the FP64 oracle: at both
+sides of the sizes that choose them (FP32 2^15 nodes and 128 columns, FP64 2^12 and 32), with
+single steps, reads and parameter changes between the blocks, and in a replayed CUDA graph.
+
+Tolerances as in test_gpu_parity.py: FP64 1e-14 a few steps on; FP32 1e-6 sqrt(n) + 1e-6.
+"""
+import ctypes
+import math
+import os
+
+import numpy as np
+import pytest
+
+from oracle import eos
+from oracle import lbm as olbm
+from paper_2301_12869_gb300 import _build, inputs, lbm
+from test_gpu_walk import T_C, read, setup, tolerance
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def cuda_lib():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    if not os.path.exists(lbm.LIB_PATH):
+        _build.build()
+    lbm.load()
+
+
+@pytest.mark.parametrize("nx, ny, precision, form, zh", [
+    (4, 8192, "fp32", 2, False), (4, 8193, "fp32", 1, False), (128, 256, "fp32", 2, True), (128, 257, "fp32", 2, False),
+    (132, 40, "fp32", 1, False), (68, 301, "fp32", 2, False), (16, 3, "fp32", 2, True), (4, 1, "fp32", 1, False),
+    (32, 128, "fp64", 2, False), (32, 129, "fp64", 1, False), (34, 60, "fp64", 2, False), (2, 2048, "fp64", 2, True),
+    (22, 186, "fp64", 1, True), (4, 1, "fp64", 2, False),
+])
+def test_blocks_and_single_steps(nx, ny, precision, form, zh):
+    p, op, rho0, f = setup(nx, ny, precision, form, zh)
+    tol = tolerance(precision, 16)
+    h = lbm.lbm_init(p, rho0)
+    try:
+        lbm.lbm_set_state(h, f)
+        f = read(h, p)
+        for block in ((5,), (1,), (2, 1, 1, 1), (1, 4)):  # the state is read after each
+            for n in block:
+                lbm.lbm_step(h, n)
+            f = olbm.run(f, op, sum(block))
+            got = read(h, p)
+            assert np.max(np.abs(got - f)) <= tol, block
+            assert lbm.lbm_reduce(h, lbm.LBM_REDUCE_MASS)[0] == pytest.approx(float(np.sum(got)), rel=1e-12)
+        rho = np.empty((ny, nx))
+        lbm.lbm_moments(h, rho)
+        assert np.max(np.abs(rho - olbm.macroscopic(f, op).rho)) <= tol
+        assert lbm.lbm_status(h) == lbm.LBM_OK
+    finally:
+        lbm.lbm_destroy(h)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_parameters_change_between_blocks(precision):
+    """To a general relaxation time (the population step), another gravity form, and back."""
+    p, op, rho0, f = setup(8, 100, precision, 2, False)
+    tol = tolerance(precision, 15)
+    h = lbm.lbm_init(p, rho0)
+    try:
+        lbm.lbm_set_state(h, f)
+        f = read(h, p)
+        for tau, form in ((1.0, 2), (0.9, 1), (1.0, 2)):
+            p.tau_nu, p.gravity_form = tau, form
+            op.tau_nu, op.form = tau, form
+            lbm.lbm_set_params(h, p)
+            lbm.lbm_step(h, 5)
+            f = olbm.run(f, op, 5)
+        assert np.max(np.abs(read(h, p) - f)) <= tol
+    finally:
+        lbm.lbm_destroy(h)
+
+
+@pytest.mark.parametrize("nx, ny, precision", [(4, 60, "fp64"), (64, 40, "fp32"), (256, 200, "fp32")])
+@pytest.mark.parametrize("before", [0, 6])
+@pytest.mark.parametrize("block", [2, 6])
+def test_captured_steps_replay(nx, ny, precision, before, block):
+    """Steps captured in a CUDA graph (an even number: two buffers take turns) and replayed, from
+    a state just set or already stepped, on the walk and on chip; then steps without the graph."""
+    import torch
+
+    p, op, rho0, f = setup(nx, ny, precision, 2, False)
+    tol = tolerance(precision, before + 3 * block + 2)
+    s = torch.cuda.Stream()
+    h = lbm.lbm_init(p, rho0, stream=s.cuda_stream)
+    try:
+        lbm.lbm_set_state(h, f)
+        f = read(h, p)
+        lbm.lbm_step(h, before)
+        if before:
+            read(h, p)  # the sums of an on-chip block are not formed until something needs them
+        g = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g, stream=s):
+            lbm.lbm_step(h, block)
+        with torch.cuda.stream(s):
+            for _ in range(3):
+                g.replay()
+        lbm.lbm_step(h, 2)
+        f = olbm.run(f, op, before + 3 * block + 2)
+        assert np.max(np.abs(read(h, p) - f)) <= tol
+    finally:
+        lbm.lbm_destroy(h)
