@@ -315,6 +315,11 @@ __global__ void __launch_bounds__(ItemOf<T>::max_threads, sizeof(T) == 4 && R > 
   __shared__ double gram_s[ACC ? NG : 1][ACC ? kColCluster * kColWarps : 1];
   __shared__ double gam_s[NU];
   __shared__ int col_s, ok_s, bad_s[kColCluster];
+  // the column's constants: double-float and FP64 ones in shared memory, where they leave registers to
+  // the arithmetic's chains (whole calls: 1024 columns double-float 13.1 -> 12.3 ms, 320 columns FP64
+  // 17.3 -> 16.8 ms; 4 x 200 FP64 4.70 -> 4.60 us a step). FP32 ones cost its chain a load: 5.84 -> 5.95 ms
+  constexpr bool SHARED_K = sizeof(T) == 8;
+  __shared__ UnitT<V> k_s;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = blockDim.x, NW = NT >> 5;
   cg::cluster_group cluster = cg::this_cluster();
@@ -365,6 +370,12 @@ __global__ void __launch_bounds__(ItemOf<T>::max_threads, sizeof(T) == 4 && R > 
       if (turn) break;
       col = a.one;
     }
+    UnitT<V> k_r{};
+    if constexpr (!SHARED_K)
+      k_r = column_unit<V>(a, col);
+    else if (tid == 0)
+      k_s = column_unit<V>(a, col);
+    const UnitT<V>& k = SHARED_K ? k_s : k_r;
     const long long t_start = [] { long long t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t; }();
     const int ny = col.ny;
     const size_t NN = size_t(nx) * ny;
@@ -372,7 +383,6 @@ __global__ void __launch_bounds__(ItemOf<T>::max_threads, sizeof(T) == 4 && R > 
     const int rows = rbase + (rank < rrem ? 1 : 0), y0 = rank * rbase + min(rank, rrem);
     const int rows_dn = rank > 0 ? rbase + (rank - 1 < rrem ? 1 : 0) : 0;  // rows of the rank below
     const int items = rows * P;
-    const UnitT<V> k = column_unit<V>(a, col);
     const bool mean = col.form == 2, zh = a.zh != 0;
     const S inv_n = mass_of<S>(1.0 / double(NN));
     T* f = static_cast<T*>(a.f) + 9 * col.node_off;
@@ -460,6 +470,7 @@ __global__ void __launch_bounds__(ItemOf<T>::max_threads, sizeof(T) == 4 && R > 
       }
     };
     if (zh) {
+      if (SHARED_K) __syncthreads();  // k
       if (mean) {
         sync();  // mass_s of the column before
         put_mass(mass_of<S>(mass0));
