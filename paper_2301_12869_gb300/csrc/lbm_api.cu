@@ -336,13 +336,17 @@ bool walk_usable(const lbm_handle* h) {
 }
 bool walk_eligible(const lbm_handle* h) { return h->tiling.variant == 0 && walk_usable(h); }
 
-// Lattices small enough for one cluster are stepped on chip, any number of steps a launch: FP32
-// up to 2^15 nodes 128 wide (64 x 128: 2.6 us a step, 4.6 walked, 6.7 on populations), FP64 up to
-// 2^12 nodes 32 wide (4 x 200: 4.7 us a step against 13.6 on populations: a node a lane is 99 FP64
-// instructions of 61 clocks, 3.1 us; beyond, the FP64 pipes of eight SMs take longer than all).
+// Lattices small enough for one cluster are stepped on chip, a call's steps in a launch: FP32 up to
+// 2^14 nodes 128 wide (64 x 128 in calls of 64 steps: 2.6 us a step, 4.7 walked, 6.7 on populations;
+// 64 x 256 3.3 and 4.6; 64 x 512 6.2 and 4.0, the eight SMs' arithmetic), FP64 up to 2^11 nodes 32
+// wide (4 x 200: 4.6 us a step against 14 on populations, 4 x 500 9.1 against 20; 24 x 125 16.4
+// against 12.9: a node a lane is 99 FP64 instructions of 61 clocks). A launch loads and stores the
+// populations, 8 to 11 us, so a call has to have some steps: FP32 64 x 256 in calls of 4 steps takes
+// 5.7 us a step and walks in 4.7, of 8 4.4 and 4.6; FP64 4 x 500 in calls of 4 steps 10.8.
+constexpr int kColumnStepsF = 8, kColumnStepsD = 4;
 bool column_fits(const lbm_params& p) {
   const long long n = (long long)p.nx * p.ny;
-  return !p.thermal && n <= (p.precision == LBM_FP32 ? 1 << 15 : 1 << 12);
+  return !p.thermal && n <= (p.precision == LBM_FP32 ? 1 << 14 : 1 << 11);
 }
 bool column_usable(const lbm_handle* h) { return h->column.ok && lbm::unit_relaxation(h->phys); }
 
@@ -725,9 +729,10 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
   if (!h) { set_err(g_err, "handle is NULL"); return LBM_EINVAL; }
   if (nsteps < 0) { set_err(h->err, "nsteps must be >= 0"); return LBM_EINVAL; }
   const bool block = nsteps + h->since_io >= kWalkSteps;  // not a single step between reads
-  if (block && h->tiling.variant == 0 && column_usable(h)) {
+  if (nsteps >= (h->p.precision == LBM_FP32 ? kColumnStepsF : kColumnStepsD) && h->tiling.variant == 0 &&
+      column_usable(h) && !(h->mom && capturing(h))) {
     if (int rc = leave_moments(h)) return rc;
-    if (nsteps > 0) h->parts_ok = false;
+    h->parts_ok = false;
     h->since_io = kWalkSteps;
     LBM_CUDA(h, column_launch(h, h->f[h->cur], nsteps));
     h->steps += nsteps;

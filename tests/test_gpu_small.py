@@ -1,5 +1,5 @@
 """Small lattices of a handle, stepped on chip a block at a time, against the FP64 oracle: at both
-sides of the sizes that choose them (FP32 2^15 nodes and 128 columns, FP64 2^12 and 32), with
+sides of the sizes that choose them (FP32 2^14 nodes and 128 columns, FP64 2^11 and 32), with
 single steps, reads and parameter changes between the blocks, and in a replayed CUDA graph.
 
 Tolerances as in test_gpu_parity.py: FP64 1e-14 a few steps on; FP32 1e-6 sqrt(n) + 1e-6.
@@ -31,19 +31,19 @@ def cuda_lib():
 
 
 @pytest.mark.parametrize("nx, ny, precision, form, zh", [
-    (4, 8192, "fp32", 2, False), (4, 8193, "fp32", 1, False), (128, 256, "fp32", 2, True), (128, 257, "fp32", 2, False),
-    (132, 40, "fp32", 1, False), (68, 301, "fp32", 2, False), (16, 3, "fp32", 2, True), (4, 1, "fp32", 1, False),
-    (32, 128, "fp64", 2, False), (32, 129, "fp64", 1, False), (34, 60, "fp64", 2, False), (2, 2048, "fp64", 2, True),
-    (22, 186, "fp64", 1, True), (4, 1, "fp64", 2, False),
+    (4, 4096, "fp32", 2, False), (4, 4097, "fp32", 1, False), (128, 128, "fp32", 2, True), (128, 129, "fp32", 2, False),
+    (132, 40, "fp32", 1, False), (68, 240, "fp32", 2, False), (16, 3, "fp32", 2, True), (4, 1, "fp32", 1, False),
+    (32, 64, "fp64", 2, False), (32, 65, "fp64", 1, False), (34, 60, "fp64", 2, False), (2, 1024, "fp64", 2, True),
+    (22, 93, "fp64", 1, True), (4, 1, "fp64", 2, False),
 ])
 def test_blocks_and_single_steps(nx, ny, precision, form, zh):
     p, op, rho0, f = setup(nx, ny, precision, form, zh)
-    tol = tolerance(precision, 16)
+    tol = tolerance(precision, 31)
     h = lbm.lbm_init(p, rho0)
     try:
         lbm.lbm_set_state(h, f)
         f = read(h, p)
-        for block in ((5,), (1,), (2, 1, 1, 1), (1, 4)):  # the state is read after each
+        for block in ((9,), (1,), (2, 1, 1, 1), (1, 8), (7,)):  # the state is read after each
             for n in block:
                 lbm.lbm_step(h, n)
             f = olbm.run(f, op, sum(block))
@@ -62,7 +62,7 @@ def test_blocks_and_single_steps(nx, ny, precision, form, zh):
 def test_parameters_change_between_blocks(precision):
     """To a general relaxation time (the population step), another gravity form, and back."""
     p, op, rho0, f = setup(8, 100, precision, 2, False)
-    tol = tolerance(precision, 15)
+    tol = tolerance(precision, 27)
     h = lbm.lbm_init(p, rho0)
     try:
         lbm.lbm_set_state(h, f)
@@ -71,16 +71,16 @@ def test_parameters_change_between_blocks(precision):
             p.tau_nu, p.gravity_form = tau, form
             op.tau_nu, op.form = tau, form
             lbm.lbm_set_params(h, p)
-            lbm.lbm_step(h, 5)
-            f = olbm.run(f, op, 5)
+            lbm.lbm_step(h, 9)
+            f = olbm.run(f, op, 9)
         assert np.max(np.abs(read(h, p) - f)) <= tol
     finally:
         lbm.lbm_destroy(h)
 
 
 @pytest.mark.parametrize("nx, ny, precision", [(4, 60, "fp64"), (64, 40, "fp32"), (256, 200, "fp32")])
-@pytest.mark.parametrize("before", [0, 6])
-@pytest.mark.parametrize("block", [2, 6])
+@pytest.mark.parametrize("before", [0, 9])
+@pytest.mark.parametrize("block", [2, 10])
 def test_captured_steps_replay(nx, ny, precision, before, block):
     """Steps captured in a CUDA graph (an even number: two buffers take turns) and replayed, from
     a state just set or already stepped, on the walk and on chip; then steps without the graph."""
