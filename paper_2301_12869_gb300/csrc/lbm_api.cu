@@ -499,6 +499,10 @@ int walk_steps(lbm_handle* h, int64_t nsteps) {
 }
 
 int run_moments(lbm_handle* h, double* rho, double* ux, double* uy) {
+  if (h->mom && rho && !ux && !uy) {
+    LBM_CUDA(h, lbm::launch_density(h->p.precision, h->phys, h->m(h->mcur), h->Tf, rho, h->N, h->status, h->stream));
+    return LBM_OK;
+  }
   if (h->mom) {
     lbm::WalkIO io = walk_io(h, h->mcur);
     io.Tfield = h->Tf;
@@ -846,16 +850,18 @@ int lbm_get_state(lbm_handle* h, double* f, int where, int64_t* steps_done) {
   if (!f || (where != LBM_HOST && where != LBM_DEVICE)) { set_err(h->err, "bad f or where"); return LBM_EINVAL; }
   if (steps_done) *steps_done = h->steps;
   if (int rc = form_populations(h)) return rc;
+  if (where == LBM_DEVICE) {
+    LBM_CUDA(h, lbm::launch_state_out(h->p.precision, h->f[h->cur], f, h->N, h->p.rho_ref, h->stream));
+    return LBM_OK;
+  }
   for (int i = 0; i < 9; ++i) {
     const void* plane = static_cast<const char*>(h->f[h->cur]) + size_t(i) * h->N * h->s;
     const double add = kWeights[i] * h->p.rho_ref;
-    double* dst = where == LBM_DEVICE ? f + size_t(i) * h->N : h->ux;  // host path stages through ux
-    LBM_CUDA(h, lbm::launch_plane_to_double(h->p.precision, plane, dst, h->N, add, h->stream));
-    if (where == LBM_HOST)
-      LBM_CUDA(h, cudaMemcpyAsync(f + size_t(i) * h->N, h->ux, h->N * sizeof(double), cudaMemcpyDeviceToHost,
-                                  h->stream));
+    // a host state is staged through ux, a plane at a time
+    LBM_CUDA(h, lbm::launch_plane_to_double(h->p.precision, plane, h->ux, h->N, add, h->stream));
+    LBM_CUDA(h, cudaMemcpyAsync(f + size_t(i) * h->N, h->ux, h->N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   }
-  return where == LBM_HOST ? device_status(h) : LBM_OK;
+  return device_status(h);
 }
 
 int lbm_set_state(lbm_handle* h, const double* f, int where, int64_t steps_done) {
@@ -865,19 +871,20 @@ int lbm_set_state(lbm_handle* h, const double* f, int where, int64_t steps_done)
   h->pop = true;
   h->mom = false;
   h->since_io = 0;
-  for (int i = 0; i < 9; ++i) {
-    void* plane = static_cast<char*>(h->f[h->cur]) + size_t(i) * h->N * h->s;
-    const double sub = kWeights[i] * h->p.rho_ref;
-    const double* src = f + size_t(i) * h->N;
-    if (where == LBM_HOST) {  // staged through ux, one plane at a time (stream-ordered)
-      LBM_CUDA(h, cudaMemcpyAsync(h->ux, src, h->N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-      src = h->ux;
+  if (where == LBM_DEVICE) {
+    LBM_CUDA(h, lbm::launch_state_in(h->p.precision, f, h->f[h->cur], h->N, h->p.rho_ref, h->parts[h->pcur], h->P,
+                                     h->stream));
+    h->npart = h->P;
+    h->parts_ok = true;
+  } else {  // staged through ux, one plane at a time (stream-ordered)
+    for (int i = 0; i < 9; ++i) {
+      void* plane = static_cast<char*>(h->f[h->cur]) + size_t(i) * h->N * h->s;
+      LBM_CUDA(h, cudaMemcpyAsync(h->ux, f + size_t(i) * h->N, h->N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+      LBM_CUDA(h, lbm::launch_plane_from_double(h->p.precision, h->ux, plane, h->N, kWeights[i] * h->p.rho_ref, h->stream));
     }
-    LBM_CUDA(h, lbm::launch_plane_from_double(h->p.precision, src, plane, h->N, sub, h->stream));
+    if (int rc = refresh_partials(h)) return rc;
   }
   LBM_CUDA(h, cudaMemsetAsync(h->status, 0, sizeof(int), h->stream));
-  int rc = refresh_partials(h);
-  if (rc) return rc;
   h->have_prev = false;
   h->steps = steps_done;
   LBM_CUDA(h, cudaStreamSynchronize(h->stream));

@@ -108,6 +108,10 @@ cudaError_t launch_walk(int precision, int mode, const WalkTiling& t, const Step
                         cudaStream_t stream);
 // M_t of the populations f*_t, and its partial sums (one per CTA of the tiling)
 cudaError_t launch_pull(int precision, const WalkTiling& t, const StepPhys& ph, const WalkIO& io, cudaStream_t stream);
+// rho of the moments (drho, j) whose first plane is dr, as doubles; Tfield as in WalkIO. Sets the
+// status of a non-physical density as the step does.
+cudaError_t launch_density(int precision, const StepPhys& ph, const void* dr, const void* Tfield, double* rho, size_t n,
+                           int* status, cudaStream_t stream);
 bool unit_relaxation(const StepPhys& p);  // every relaxation time 1
 
 // initial state and the FP64 partial sums of its stored values into part[0..npart)
@@ -122,6 +126,10 @@ cudaError_t launch_plane_to_double(int precision, const void* plane, double* out
                                    cudaStream_t stream);
 cudaError_t launch_plane_from_double(int precision, const double* in, void* plane, size_t n, double sub,
                                      cudaStream_t stream);
+// a whole state of n nodes: f = in - w_i rho_ref with the partial sums of f / out = f + w_i rho_ref
+cudaError_t launch_state_in(int precision, const double* in, void* f, size_t n, double rho_ref, double* part, int npart,
+                            cudaStream_t stream);
+cudaError_t launch_state_out(int precision, const void* f, double* out, size_t n, double rho_ref, cudaStream_t stream);
 // max |a - b| over n (b may be NULL: max |a|); max sqrt(ux^2+uy^2)
 cudaError_t launch_max_abs_diff(const double* a, const double* b, size_t n, double* out, cudaStream_t stream);
 cudaError_t launch_max_speed(const double* ux, const double* uy, size_t n, double* out, cudaStream_t stream);

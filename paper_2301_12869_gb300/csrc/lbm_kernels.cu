@@ -725,7 +725,7 @@ struct Quad<float> {
   }
   // store d rounded to FP32 and return the stored values as pairs
   __device__ static void store(float* p, const double (&d)[4], V (&v)[2]) {
-    const float4 q = make_float4(float(d[0]), float(d[1]), float(d[2]), float(d[3]));
+    const float4 q = make_float4(narrow(d[0]), narrow(d[1]), narrow(d[2]), narrow(d[3]));
     *reinterpret_cast<float4*>(p) = q;
     v[0] = make_f2(q.x, q.y);
     v[1] = make_f2(q.z, q.w);
@@ -823,17 +823,94 @@ __global__ void sum_partials_kernel(const double* part, int npart, double* out) 
   if (threadIdx.x == 0) out[0] = s;
 }
 
+// ---- a whole state in absolute FP64 values [9][n] <-> the stored deviations g_i = f_i - w_i rho_ref,
+// two nodes a thread and plane (16 bytes of the caller's array, so that a warp's accesses are whole
+// lines), all planes in one launch. In: with the FP64 partial sums of the stored values, as
+// partials_kernel adds them. VEC: the caller's array starts on a 16-byte boundary. 1024 x 4096 nodes,
+// cold: in 201 us (nine launches and the sums' pass) -> 108 in FP32, 202 -> 159 in FP64 (its 18 FP64
+// additions a node); out 169 -> 155 and 118 -> 92. 256 x 768, where the launches count: whole pass of
+// 200 steps with both and the density 1293 -> 1241 us
+constexpr int kStateThreads = 512;
+template <typename T>
+struct Two;
+template <>
+struct Two<float> {
+  using type = float2;
+  __device__ static void add(Acc<f2>& acc, float2 v, int i) { acc.add(make_f2(v.x, v.y), i); }
+};
+template <>
+struct Two<double> {
+  using type = double2;
+  __device__ static void add(Acc<double>& acc, double2 v, int i) {
+    acc.add(v.x, i);
+    acc.add(v.y, i);
+  }
+};
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(kStateThreads, 2) state_in_kernel(const double* __restrict__ in, T* __restrict__ f,
+                                                                    size_t n, double rho_ref,
+                                                                    double* __restrict__ part) {
+  using T2 = typename Two<T>::type;
+  const size_t groups = n / 2;
+  const size_t chunk = (groups + gridDim.x - 1) / gridDim.x;
+  const size_t k0 = blockIdx.x * chunk, k1 = min(groups, k0 + chunk);
+  Acc<typename Quad<T>::V> acc;
+  for (size_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
+    double2 d[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const double* src = in + i * n + 2 * k;
+      if constexpr (VEC)
+        d[i] = *reinterpret_cast<const double2*>(src);
+      else
+        d[i] = make_double2(src[0], src[1]);
+    }
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const double sub = __dmul_rn(w_of(i), rho_ref);
+      T2 v;
+      v.x = narrow_to(d[i].x - sub, T{});
+      v.y = narrow_to(d[i].y - sub, T{});
+      *reinterpret_cast<T2*>(f + i * n + 2 * k) = v;
+      Two<T>::add(acc, v, i % 3);
+    }
+  }
+  block_partial(acc, part);
+}
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(kStateThreads, 2) state_out_kernel(const T* __restrict__ f, double* __restrict__ out,
+                                                                     size_t n, double rho_ref) {
+  using T2 = typename Two<T>::type;
+  for (size_t k = blockIdx.x * size_t(blockDim.x) + threadIdx.x; k < n / 2; k += size_t(gridDim.x) * blockDim.x) {
+    T2 v[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) v[i] = *reinterpret_cast<const T2*>(f + i * n + 2 * k);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const double add = __dmul_rn(w_of(i), rho_ref);
+      const double2 d = make_double2(widen(v[i].x) + add, widen(v[i].y) + add);
+      double* dst = out + i * n + 2 * k;
+      if constexpr (VEC) {
+        *reinterpret_cast<double2*>(dst) = d;
+      } else {
+        dst[0] = d.x;
+        dst[1] = d.y;
+      }
+    }
+  }
+}
+
 // one population plane: out[q] = plane[q] + add  /  plane[q] = in[q] - sub
 template <typename T>
 __global__ void plane_to_double_kernel(const T* __restrict__ plane, double* __restrict__ out, size_t n, double add) {
   for (size_t q = blockIdx.x * size_t(blockDim.x) + threadIdx.x; q < n; q += size_t(gridDim.x) * blockDim.x)
-    out[q] = double(plane[q]) + add;
+    out[q] = widen(plane[q]) + add;
 }
 
 template <typename T>
 __global__ void plane_from_double_kernel(const double* __restrict__ in, T* __restrict__ plane, size_t n, double sub) {
   for (size_t q = blockIdx.x * size_t(blockDim.x) + threadIdx.x; q < n; q += size_t(gridDim.x) * blockDim.x)
-    plane[q] = T(in[q] - sub);
+    plane[q] = narrow_to(in[q] - sub, T{});
 }
 
 // non-negative doubles order like their bit patterns; NaN (0x7ff8...) sorts above +inf
@@ -1168,6 +1245,40 @@ cudaError_t launch_plane_from_double(int precision, const double* in, void* plan
     plane_from_double_kernel<float><<<grid_for(n, 256), 256, 0, stream>>>(in, static_cast<float*>(plane), n, sub);
   else
     plane_from_double_kernel<double><<<grid_for(n, 256), 256, 0, stream>>>(in, static_cast<double*>(plane), n, sub);
+  return cudaGetLastError();
+}
+
+namespace {
+bool on_16_bytes(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+template <typename T>
+void state_in(const double* in, void* f, size_t n, double rho_ref, double* part, int npart, cudaStream_t s) {
+  if (on_16_bytes(in))
+    state_in_kernel<T, true><<<npart, kStateThreads, 0, s>>>(in, static_cast<T*>(f), n, rho_ref, part);
+  else
+    state_in_kernel<T, false><<<npart, kStateThreads, 0, s>>>(in, static_cast<T*>(f), n, rho_ref, part);
+}
+template <typename T>
+void state_out(const void* f, double* out, size_t n, double rho_ref, cudaStream_t s) {
+  const unsigned grid = grid_for(n / 2, kStateThreads);
+  if (on_16_bytes(out))
+    state_out_kernel<T, true><<<grid, kStateThreads, 0, s>>>(static_cast<const T*>(f), out, n, rho_ref);
+  else
+    state_out_kernel<T, false><<<grid, kStateThreads, 0, s>>>(static_cast<const T*>(f), out, n, rho_ref);
+}
+}  // namespace
+cudaError_t launch_state_in(int precision, const double* in, void* f, size_t n, double rho_ref, double* part, int npart,
+                            cudaStream_t stream) {
+  if (precision == 1)
+    state_in<float>(in, f, n, rho_ref, part, npart, stream);
+  else
+    state_in<double>(in, f, n, rho_ref, part, npart, stream);
+  return cudaGetLastError();
+}
+cudaError_t launch_state_out(int precision, const void* f, double* out, size_t n, double rho_ref, cudaStream_t stream) {
+  if (precision == 1)
+    state_out<float>(f, out, n, rho_ref, stream);
+  else
+    state_out<double>(f, out, n, rho_ref, stream);
   return cudaGetLastError();
 }
 

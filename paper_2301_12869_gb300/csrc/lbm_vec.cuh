@@ -147,4 +147,34 @@ __device__ __forceinline__ double hsum(double x) { return x; }
 __device__ __forceinline__ double hsum(float x) { return double(x); }
 __device__ __forceinline__ double hsum(f2 x) { return double(lo(x)) + double(hi(x)); }
 
+// FP64 <-> FP32 conversions share the slow FP64 pipe with the additions (2 lanes a clock and SM), so
+// for a whole state they cost more than its memory traffic. These form the same values with integer
+// instructions; zero, infinities, NaN and what is denormal in FP32 take the conversion (volatile: it
+// stays behind its branch instead of being executed for every value and selected).
+__device__ __forceinline__ float narrow(double d) {  // to the nearest FP32, ties to even
+  const uint32_t h = uint32_t(__double2hiint(d)), l = uint32_t(__double2loint(d));
+  const uint32_t e = (h >> 20) & 0x7ffu;
+  if (e - 897u >= 253u) {  // 2^-126 <= |d| < 2^127 otherwise
+    float r;
+    asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(r) : "d"(d));
+    return r;
+  }
+  uint32_t m = ((h & 0x7fffffffu) - (896u << 20)) << 3 | l >> 29;  // exponent and 23 bits, truncated
+  m += ((l & 0x1fffffffu) + 0x0fffffffu + (m & 1u)) >> 29;          // the 29 bits below round it
+  return __uint_as_float(m | (h & 0x80000000u));
+}
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t b = __float_as_uint(f);
+  const uint32_t e = (b >> 23) & 0xffu;
+  if (e - 1u >= 254u) {
+    double r;
+    asm volatile("cvt.f64.f32 %0, %1;" : "=d"(r) : "f"(f));
+    return r;
+  }
+  return __hiloint2double(int((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), int(b << 29));
+}
+__device__ __forceinline__ double narrow_to(double d, double) { return d; }
+__device__ __forceinline__ float narrow_to(double d, float) { return narrow(d); }
+__device__ __forceinline__ double widen(double d) { return d; }
+
 }  // namespace lbm

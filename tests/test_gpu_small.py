@@ -5,15 +5,13 @@ single steps, reads and parameter changes between the blocks, and in a replayed 
 Tolerances as in test_gpu_parity.py: FP64 1e-14 a few steps on; FP32 1e-6 sqrt(n) + 1e-6.
 """
 import ctypes
-import math
 import os
 
 import numpy as np
 import pytest
 
-from oracle import eos
 from oracle import lbm as olbm
-from paper_2301_12869_gb300 import _build, inputs, lbm
+from paper_2301_12869_gb300 import _build, lbm
 from test_gpu_walk import T_C, read, setup, tolerance
 
 pytestmark = pytest.mark.gpu
@@ -106,5 +104,81 @@ def test_captured_steps_replay(nx, ny, precision, before, block):
         lbm.lbm_step(h, 2)
         f = olbm.run(f, op, before + 3 * block + 2)
         assert np.max(np.abs(read(h, p) - f)) <= tol
+    finally:
+        lbm.lbm_destroy(h)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_state_in_and_out_keep_every_value(precision, offset):
+    """Device states on 16- and 8-byte boundaries: each value minus its share of the reference,
+    rounded once to the storage type - ties, denormals, infinities and NaN among them - and back."""
+    import torch
+
+    nx, ny = 64, 37
+    n = nx * ny
+    rho_ref = 0.0 if offset else 0.173
+    rng = np.random.default_rng(5)
+    with np.errstate(over="ignore", under="ignore", invalid="ignore"):
+        v = rng.normal(size=9 * n) * np.exp2(rng.integers(-160, 132, 9 * n))
+        half = np.float32(rng.normal(size=n)).astype(np.float64)  # halfway between two FP32 values
+        v[:n] = half + np.float64(np.spacing(np.float32(half))) / 2
+        v[n:n + 12] = [0.0, -0.0, np.inf, -np.inf, np.nan, 2.0**-126, -2.0**-126 * (1 - 2.0**-25), 2.0**-149, 2.0**-150,
+                       3.4028235677973366e38, 2.0**127, 1 - 2.0**-26]
+        raw = torch.zeros(9 * n + 1, dtype=torch.float64, device="cuda")
+        src = raw[offset:offset + 9 * n]
+        src.copy_(torch.from_numpy(v))
+        assert src.data_ptr() % 16 == 8 * offset
+        w = np.repeat(np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4), n) * rho_ref
+        want = v - w
+        if precision == "fp32":
+            want = want.astype(np.float32).astype(np.float64)
+        want = want + w
+    h = lbm.lbm_init(lbm.make_params(nx, ny, 0.85 * T_C, precision, a=0.25, rho_ref=rho_ref), np.full((ny, nx), 0.1))
+    out = torch.zeros(9 * n + 1, dtype=torch.float64, device="cuda")[offset:offset + 9 * n]
+    try:
+        lib = lbm.load()
+        assert lib.lbm_set_state(h, ctypes.c_void_p(src.data_ptr()), lbm.LBM_DEVICE, 0) == lbm.LBM_OK
+        assert lib.lbm_get_state(h, ctypes.c_void_p(out.data_ptr()), lbm.LBM_DEVICE, None) == lbm.LBM_OK
+        torch.cuda.synchronize()
+        got = out.cpu().numpy()
+    finally:
+        lbm.lbm_destroy(h)
+    assert np.array_equal(got, want, equal_nan=True)
+
+
+@pytest.mark.parametrize("thermal", [0, 1])
+def test_density_alone_is_the_density_with_the_velocity(thermal):
+    """rho of a state held as moments, without the stencil and with it."""
+    nx, ny = 256, 257
+    kw = dict(thermal=1, T_bot=0.9 * T_C, T_top=0.8 * T_C) if thermal else {}
+    p, _, rho0, f = setup(nx, ny, "fp64", 1, False, **kw)
+    h = lbm.lbm_init(p, rho0)
+    try:
+        lbm.lbm_set_state(h, f)
+        lbm.lbm_step(h, 6)
+        rho, rho2, ux = np.empty((ny, nx)), np.empty((ny, nx)), np.empty((ny, nx))
+        lbm.lbm_moments(h, rho)
+        lbm.lbm_moments(h, rho2, ux)
+        assert np.array_equal(rho, rho2)
+    finally:
+        lbm.lbm_destroy(h)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("factor, code", [(1.0, lbm.LBM_OK), (40.0, lbm.LBM_ENONPHYS)])
+def test_density_alone_reports_what_psi_would(precision, factor, code):
+    """A temperature at which p_EOS > rho/3 is set under a state held as moments: psi^2 < 0 is
+    reported by rho alone, before any step."""
+    nx, ny = 256, 257
+    p, _, rho0, f = setup(nx, ny, precision, 1, False, thermal=1, T_bot=0.9 * T_C, T_top=0.8 * T_C)
+    h = lbm.lbm_init(p, rho0)
+    try:
+        lbm.lbm_set_state(h, f)
+        lbm.lbm_step(h, 6)
+        lbm.lbm_set_temperature(h, np.full((ny, nx), 0.85 * T_C * factor))
+        rho = np.empty((ny, nx))
+        rc = lbm.load().lbm_moments(h, rho.ctypes.data_as(ctypes.c_void_p), None, None, lbm.LBM_HOST)
+        assert rc == code and np.all(rho > 0)
     finally:
         lbm.lbm_destroy(h)
