@@ -44,20 +44,22 @@ GY = -1e-4
 LIQUID_ROWS = 2048
 NOISE = 1e-3
 SEED = 20230130
-BYTES_PER_NODE = {"fp32": 72, "fp64": 144}   # 9 populations read + 9 written
-# The FP64 step is bound by GB300's FP64 pipe, not by HBM: ncu counts 57 DFMA + 54 DADD +
-# 35 DMUL per node (step_kernel<double>, 1024 x 4096, tau = 1) = 203 FP64 flops per node
+BYTES_PER_NODE = {"fp32": 24, "fp64": 48}        # a handle's step: rho and j read and written
+SLAB_BYTES_PER_NODE = {"fp32": 72, "fp64": 144}  # a slab's step: 9 populations read, 9 written
+# The FP64 step is bound by GB300's FP64 pipe, not by HBM: ncu counts 45 DFMA + 31 DADD +
+# 25 DMUL a node (walk_kernel<double>, 1024 x 4096, tau = 1), 1.16 times the 87 instructions a
+# node's own arithmetic takes (the rest is the strips' halo): 145 / 1.16 = 125 FP64 flops a node
 # (FMA = 2). Peak: 2 FP64 FMAs per SM per clock, the rate the nominal 1.25 TFLOP/s dense
 # FP64 of GB300 gives for 152 SMs at 2.07 GHz (1.25e12 / (2 x 152 x 2.07e9) = 1.99).
-FP64_FLOPS_PER_NODE = 203
+FP64_FLOPS_PER_NODE = 125
 FP64_PEAK_TFLOPS = 2 * 2 * 152 * 2.07e9 / 1e12
 # With (rho - <rho>) g at g_y = -1e-4 the 2048-row vapour column accelerates freely
 # (max |u| = 0.42 after 500 steps, NaN before 1000): the workload is physical only for
 # its first ~500 steps. Timed runs longer than WINDOW steps restore the post-warm-up
 # state every WINDOW steps (lbm_set_state from a device snapshot, inside the timing).
 WINDOW = 400
-KERNEL_SRC = os.path.join(ROOT, "paper_2301_12869_gb300", "csrc", "lbm_kernels.cu")
-PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "step_kernel_fp32_1024x4096.json")
+KERNEL_SRC = os.path.join(ROOT, "paper_2301_12869_gb300", "csrc", "lbm_walk.cu")
+PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "walk_kernel_fp32_1024x4096.json")
 
 
 PREROLL_CYCLES = 200_000  # ~0.1 ms at 2 GHz
@@ -931,10 +933,10 @@ def time_to_steady(args, lbm, inputs, world, rank, torch):
 # ---------------------------------------------------------------- thermal variant
 TH_NX, TH_NY, TH_LIQUID = 512, 2048, 1024
 TH_TBOT, TH_TTOP, TH_GY = 0.95, 0.80, -5e-5
-# per node and step, as launched: fused step 72 B populations + 4 B T read, 12 B rho/u
+# per node and step, as launched: fused step 24 B moments + 4 B T read, 12 B rho/u
 # written; Heun kernel 4 B T + 12 B rho/u read, 4 B T written (FP32 storage, rho and u
 # handed over as floats; FP64 storage doubles every term)
-TH_BYTES_PER_NODE = {"fp32": 88 + 20, "fp64": 176 + 40}
+TH_BYTES_PER_NODE = {"fp32": 40 + 20, "fp64": 80 + 40}
 # The heated column goes non-physical: its 1024 vapour rows weigh more than the vapour's
 # saturation pressure can carry at g_y = -5e-5 (scale height of the vapour ~100 rows), so
 # the vapour falls freely and the top empties (max |u| = |g| t) within ~5000 steps. Timed
@@ -1508,7 +1510,7 @@ def main(argv=None):
         ms, units = aggregate(local_ms, local_units, torch)
         value = units / (ms / 1e3) / 1e6
         kernel_s = ms / 1e3 / args.steps  # the slowest rank's step, exchanges included
-        alg_bytes = BYTES_PER_NODE[args.precision] * NX * sl.ny_own
+        alg_bytes = SLAB_BYTES_PER_NODE[args.precision] * NX * sl.ny_own
         achieved = alg_bytes / kernel_s / 1e9
         mass = e2e["mass"] if e2e else None
         info = {"column_rows": ny_total, "slab_rows_rank0": sl.ny_own, "ghost_rows_per_side": 2,
@@ -1567,9 +1569,8 @@ def main(argv=None):
         del snapshot
         torch.cuda.empty_cache()
         scaling, parallelism = "weak", (f"replicas x{world}" if world > 1 else "single GPU")
-        launches = args.steps + restores * (9 + 1)
-        kernel_name = (f"step_kernel_ws<8 consumer warps, {info['stages']} stages>" if args.precision == "fp32"
-                       else "step_kernel<double, 128-node bands>")
+        launches = args.steps + restores * (9 + 1 + 1)
+        kernel_name = "walk_kernel<float>" if args.precision == "fp32" else "walk_kernel<double>"
     # the metric's second half: time to steady state of the batched columns (all ranks, each
     # on its share of the columns)
     steady = None if args.no_steady else time_to_steady(args, lbm, inputs, world, rank, torch)
@@ -1580,6 +1581,7 @@ def main(argv=None):
         if world > 1:
             torch.distributed.destroy_process_group()
         return 0
+    fp64_nodes = alg_bytes / (SLAB_BYTES_PER_NODE if use_slabs else BYTES_PER_NODE)["fp64"]
     line = {
         "metric": "MLUPS", "value": value, "unit": "MLUPS", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": scaling,
@@ -1595,9 +1597,9 @@ def main(argv=None):
             "frac": achieved / peaks["hbm_gbs"], "traffic": None if use_slabs else traffic_from_profile(args.precision),
             "peak_kind": peak_kind, "kernel": kernel_name, "algorithmic_bytes_per_launch": alg_bytes,
         } if args.precision == "fp32" else {
-            "bound": "alu", "achieved": FP64_FLOPS_PER_NODE * alg_bytes / BYTES_PER_NODE["fp64"] / kernel_s / 1e12,
+            "bound": "alu", "achieved": FP64_FLOPS_PER_NODE * fp64_nodes / kernel_s / 1e12,
             "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": FP64_FLOPS_PER_NODE * alg_bytes / BYTES_PER_NODE["fp64"] / kernel_s / 1e12 / FP64_PEAK_TFLOPS,
+            "frac": FP64_FLOPS_PER_NODE * fp64_nodes / kernel_s / 1e12 / FP64_PEAK_TFLOPS,
             "traffic": None, "peak_kind": "derived from the nominal FP64 rate (2 FP64 FMA / SM / clock)",
             "kernel": kernel_name, "fp64_flops_per_node": FP64_FLOPS_PER_NODE,
             "hbm": {"achieved_GB_per_s": achieved, "frac_of_measured": achieved / peaks["hbm_gbs"]},
