@@ -149,16 +149,14 @@ __device__ __forceinline__ double hsum(f2 x) { return double(lo(x)) + double(hi(
 
 // FP64 <-> FP32 conversions share the slow FP64 pipe with the additions (2 lanes a clock and SM), so
 // for a whole state they cost more than its memory traffic. These form the same values with integer
-// instructions; zero, infinities, NaN and what is denormal in FP32 take the conversion (volatile: it
-// stays behind its branch instead of being executed for every value and selected).
+// instructions; zero, infinities, NaN and what is denormal in FP32 take the conversion, out of line:
+// inline it was issued for every value, if only predicated off (a 1024 x 4096 state in and out 65 us more).
+static __device__ __noinline__ float narrow_slowly(double d) { return float(d); }
+static __device__ __noinline__ double widen_slowly(float f) { return double(f); }
 __device__ __forceinline__ float narrow(double d) {  // to the nearest FP32, ties to even
   const uint32_t h = uint32_t(__double2hiint(d)), l = uint32_t(__double2loint(d));
   const uint32_t e = (h >> 20) & 0x7ffu;
-  if (e - 897u >= 253u) {  // 2^-126 <= |d| < 2^127 otherwise
-    float r;
-    asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(r) : "d"(d));
-    return r;
-  }
+  if (e - 897u >= 253u) return narrow_slowly(d);  // 2^-126 <= |d| < 2^127 otherwise
   uint32_t m = ((h & 0x7fffffffu) - (896u << 20)) << 3 | l >> 29;  // exponent and 23 bits, truncated
   m += ((l & 0x1fffffffu) + 0x0fffffffu + (m & 1u)) >> 29;          // the 29 bits below round it
   return __uint_as_float(m | (h & 0x80000000u));
@@ -166,11 +164,7 @@ __device__ __forceinline__ float narrow(double d) {  // to the nearest FP32, tie
 __device__ __forceinline__ double widen(float f) {
   const uint32_t b = __float_as_uint(f);
   const uint32_t e = (b >> 23) & 0xffu;
-  if (e - 1u >= 254u) {
-    double r;
-    asm volatile("cvt.f64.f32 %0, %1;" : "=d"(r) : "f"(f));
-    return r;
-  }
+  if (e - 1u >= 254u) return widen_slowly(f);
   return __hiloint2double(int((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), int(b << 29));
 }
 __device__ __forceinline__ double narrow_to(double d, double) { return d; }
