@@ -84,7 +84,9 @@ def workload_config(precision):
         "workload": f"single liquid column {NX}x{NY} D2Q9, {precision.upper()} populations, FP64 reductions",
         "nx": NX, "ny": NY, "T_over_Tc": TR, "a": A, "b": B, "R": R, "gravity": "(rho-<rho>)g", "g_y": GY,
         "liquid_rows": LIQUID_ROWS, "noise": NOISE, "seed": SEED, "tau": 1.0, "sigma": 1.385,
-        "l2": "state 302 MB (FP32) > 129 MB L2: no flush needed",
+        "l2": "populations 2 x 151 MB (FP32) > 129 MB L2; the step's own working set with every tau = 1 is two "
+              "50 MB buffers of moments, which stay partly in L2 from step to step as in a run (no flush; a "
+              "launch on a flushed L2 takes 26.8 us under ncu)",
         "physical_window": f"state restored from the post-warm-up snapshot every {WINDOW} steps "
                            "(the workload goes non-physical after ~500 steps)",
     }
