@@ -144,6 +144,7 @@ struct lbm_handle {
   // m(0), m(1) lie in f[1 - cur]; parts[b] holds the partial sums of m(b) while mom is set, and
   // the populations f[cur] can be formed from m(1 - mcur), the state before the last step.
   lbm::WalkTiling walk{};
+  bool walk_fits = false;  // its grid has a slot of the partial sums for every CTA
   bool pop = true, mom = false;
   int mcur = 0;
   bool parts_ok = true;  // parts[pcur] are the partial sums of f[cur] (when not mom)
@@ -332,7 +333,7 @@ constexpr int kWalkSteps = 4;
 // 2^16 nodes keep the population step: a walk's row takes 5 us of one warp's FP64 instructions
 // (4 x 200: 31.6 us a step against 13.6; 256 x 256: 48.6 against 52.1).
 bool walk_usable(const lbm_handle* h) {
-  return lbm::unit_relaxation(h->phys) && (h->p.precision == LBM_FP32 || h->N >= (size_t(1) << 16));
+  return h->walk_fits && lbm::unit_relaxation(h->phys) && (h->p.precision == LBM_FP32 || h->N >= (size_t(1) << 16));
 }
 bool walk_eligible(const lbm_handle* h) { return h->tiling.variant == 0 && walk_usable(h); }
 
@@ -652,7 +653,7 @@ int lbm_init(const lbm_params* p, const double* rho0, int rho0_where, void* stre
     h->column = lbm::plan_columns(p->precision, p->nx, p->ny, p->ny, 8, p->precision == LBM_FP32 ? 0 : 64);
     if (h->column.ok) h->column.ok = lbm::column_clusters(p->precision, h->column, false) > 0;
   }
-  lbm::plan_walk(p->precision, p->nx, p->ny, p->wall == LBM_WALL_ZOU_HE, h->nsm, h->Pcap, &h->walk);
+  h->walk_fits = lbm::plan_walk(p->precision, p->nx, p->ny, p->wall == LBM_WALL_ZOU_HE, h->nsm, h->Pcap, &h->walk);
   const Layout L = layout_for(*p, h->Pcap);
   if (p->workspace) {
     if (p->workspace_bytes < L.total || (reinterpret_cast<uintptr_t>(p->workspace) & 255)) {

@@ -102,8 +102,9 @@ struct WalkIO {
   void *rho_T, *ux_T, *uy_T;          // thermal step: this step's rho, u as reals [y][x]
   const void* Tfield;     // thermal: real[ny][nx] (NULL: uniform T)
 };
-// the tiling of a lattice on a GPU of nsm SMs; at most max_ctas CTAs (partial sums)
-void plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, WalkTiling* t);
+// the tiling of a lattice on a GPU of nsm SMs; at most max_ctas CTAs (partial sums), false where
+// that cannot be kept: such a tiling is not launched
+bool plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, WalkTiling* t);
 cudaError_t launch_walk(int precision, int mode, const WalkTiling& t, const StepPhys& ph, const WalkIO& io,
                         cudaStream_t stream);
 // M_t of the populations f*_t, and its partial sums (one per CTA of the tiling)

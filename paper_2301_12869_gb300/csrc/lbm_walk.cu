@@ -510,7 +510,7 @@ __global__ void __launch_bounds__(256) density_kernel(const DensityT<T> k, doubl
 // 0.50 with 16; an FP64 row is bound by the SM's FP64 pipe (1.57 us a warp: 100 issue slots of
 // 15.4 clocks a column) and takes 5 us alone. 1024 x 4096 FP32: 31-row strips, one wave of
 // 16 warps per SM, 22.5 us; 30 rows (two waves) 41 us, 50 rows (10 warps per SM) 27.6 us.
-void plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, WalkTiling* t) {
+bool plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, WalkTiling* t) {
   const bool fp32 = precision == 1;
   const int W = fp32 ? kColumns<float> : kColumns<double>;
   t->nx = nx;
@@ -553,8 +553,16 @@ void plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, Wa
     }
   }
   set_rows(best_h);
-  // the partial sums' slots bound the grid
+  // the partial sums' slots bound the grid: taller strips, and where a strip is the whole height
+  // (wide lattices of a few rows: 4096 x 8 FP32 has 64 slots for 69 warps) more warps a CTA
   while (t->ctas > max_ctas && t->strip_h < ny) set_rows(std::min(ny, t->strip_h + std::max(1, t->strip_h / 8)));
+  if (t->ctas > max_ctas && max_ctas > 0) {
+    const long warps = (long(t->nstrips) * t->nbands * t->seg + 31) / 32;
+    const int per_cta = int(std::min<long>(most_warps, (warps + max_ctas - 1) / max_ctas));
+    t->threads = 32 * per_cta;
+    t->ctas = int((warps + per_cta - 1) / per_cta);
+  }
+  return t->ctas <= max_ctas;
 }
 
 namespace {
