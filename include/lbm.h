@@ -131,7 +131,9 @@ int lbm_init(const lbm_params* p, const double* rho0, int rho0_where, void* stre
  * one launch of a fused kernel - with every relaxation time 1 and the default tile one that
  * holds the state between calls as rho and j of the streamed populations, from which the
  * populations are formed when they are read; a call of several steps on a small lattice is one
- * launch that keeps the lattice on chip. A step: stream (and, with Zou-He walls, rebuild the wall nodes'
+ * launch that keeps the lattice on chip. Calls captured in a CUDA graph (an even number of steps a
+ * graph) may be mixed with direct ones; from the first captured call on a handle's steps that are not
+ * on chip are those on populations. A step: stream (and, with Zou-He walls, rebuild the wall nodes'
  * incoming populations), rho, psi, <rho>, F_int, F_g, u, MRT + Li forcing, store. Device-side faults (non-physical state, timeouts) are recorded in a
  * sticky status returned by the next synchronising call.
  * Thermal variant: psi uses R T(x) of the current temperature field T^n, and the step

@@ -128,7 +128,7 @@ struct lbm_handle {
   int npart = 0;         // partials in parts[pcur]
   int P = 0;             // CTAs of the current step launch (= partials it writes)
   int Pcap = 0;          // partial slots per buffer (largest grid over the tile variants)
-  int* status = nullptr;
+  int* status = nullptr; // device status word; status[1]: `pending`, below
   double* red = nullptr; // small device outputs
   double* rho_now = nullptr;
   double* rho_prev = nullptr;
@@ -150,6 +150,14 @@ struct lbm_handle {
   bool parts_ok = true;  // parts[pcur] are the partial sums of f[cur] (when not mom)
   lbm::ColumnPlan column{};  // a small lattice is stepped on chip (ok: it fits)
   int since_io = 0;      // population steps since the populations were last set or read
+  // What a stream capture records runs at every replay, without the host's knowledge, so none of the
+  // flags above may depend on it: from the first captured call on the populations f[cur] are the only
+  // form, and parts[pcur] their sums after every call, as the calls in a graph find and leave them. A
+  // state held as moments alone when a capture began becomes populations once, by the first replay or
+  // direct call to come: the device word `pending` says whether that has yet to happen.
+  bool graphs = false;
+  int* pending() const { return status + 1; }
+  lbm::StepPhys made{};  // parameters of the step that made the moments: the populations belong to them
   void* m(int b) const { return static_cast<char*>(f[1 - cur]) + size_t(3 * b) * N * s; }
   double* mean(int b) const { return red + 4 + b; }  // Zou-He: <rho> - rho_ref for the collision of m(b)
   lbm::StepTiling tiling{};
@@ -222,7 +230,7 @@ Layout layout_for(const lbm_params& p, int P) {
   L.f1 = take(9 * N * s);
   L.parts0 = take(size_t(P) * 8);
   L.parts1 = take(size_t(P) * 8);
-  L.status = take(sizeof(int));
+  L.status = take(2 * sizeof(int));
   L.red = take(8 * sizeof(double));
   L.rho_now = take(N * 8);
   L.rho_prev = take(N * 8);
@@ -333,7 +341,8 @@ constexpr int kWalkSteps = 4;
 // 2^16 nodes keep the population step: a walk's row takes 5 us of one warp's FP64 instructions
 // (4 x 200: 31.6 us a step against 13.6; 256 x 256: 48.6 against 52.1).
 bool walk_usable(const lbm_handle* h) {
-  return h->walk_fits && lbm::unit_relaxation(h->phys) && (h->p.precision == LBM_FP32 || h->N >= (size_t(1) << 16));
+  return !h->graphs && h->walk_fits && lbm::unit_relaxation(h->phys) &&
+         (h->p.precision == LBM_FP32 || h->N >= (size_t(1) << 16));
 }
 bool walk_eligible(const lbm_handle* h) { return h->tiling.variant == 0 && walk_usable(h); }
 
@@ -373,8 +382,7 @@ cudaError_t column_launch(lbm_handle* h, void* f, int64_t nsteps) {
   return e;
 }
 
-// a stream capture in progress: what is launched runs at every replay, so the form of the state
-// must not change with it
+// a stream capture in progress: what is launched runs at every replay, not now
 bool capturing(const lbm_handle* h) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
@@ -424,24 +432,47 @@ int form_moments(lbm_handle* h) {
 }
 
 // the populations f[cur] of a state held as moments: the collision of the state before
-int form_populations(lbm_handle* h) {
-  h->since_io = 0;
-  if (h->pop) return LBM_OK;
+int launch_populations(lbm_handle* h, const int* pending) {
   lbm::WalkIO io = walk_io(h, 1 - h->mcur);
   io.fout = h->f[h->cur];
   io.Tfield = h->Tnext;  // the temperature that step used
-  LBM_CUDA(h, lbm::launch_walk(h->p.precision, lbm::WALK_POPULATIONS, h->walk, h->phys, io, h->stream));
-  h->pop = !capturing(h);  // a captured launch has not run: the moments stay the state
+  io.pending = pending;
+  LBM_CUDA(h, lbm::launch_walk(h->p.precision, lbm::WALK_POPULATIONS, h->walk, h->made, io, h->stream));
+  return LBM_OK;
+}
+
+// First in every call that reads or steps the state: a captured one, and all after it, find the state as
+// populations (see `graphs`)
+int settle(lbm_handle* h) {
+  const bool captured = capturing(h);
+  if (!captured && !h->graphs) return LBM_OK;
+  h->graphs = true;
+  if (!h->mom) return LBM_OK;
+  if (!h->pop) {
+    if (int rc = launch_populations(h, h->pending())) return rc;
+    LBM_CUDA(h, cudaMemsetAsync(h->pending(), 0, sizeof(int), h->stream));
+  }
+  h->parts_ok = false;
+  if (captured && !h->pop) return LBM_OK;  // not done yet: a direct call asks again
+  h->pop = true;
+  h->mom = false;
+  return LBM_OK;
+}
+
+int form_populations(lbm_handle* h) {
+  h->since_io = 0;
+  if (int rc = settle(h)) return rc;
+  if (h->graphs || h->pop) return LBM_OK;
+  if (int rc = launch_populations(h, nullptr)) return rc;
+  h->pop = true;
   return LBM_OK;
 }
 
 // the state as populations alone, with their partial sums
 int leave_moments(lbm_handle* h) {
-  if (!h->mom) return LBM_OK;
-  int rc = form_populations(h);
-  if (rc) return rc;
+  if (int rc = form_populations(h)) return rc;
+  if (h->graphs || !h->mom) return LBM_OK;
   h->mom = false;
-  h->pop = true;
   return refresh_partials(h);
 }
 
@@ -489,6 +520,7 @@ int walk_launch(lbm_handle* h) {
 int walk_steps(lbm_handle* h, int64_t nsteps) {
   if (nsteps == 0) return LBM_OK;
   if (int rc = form_moments(h)) return rc;
+  h->made = h->phys;
   for (int64_t t = 0; t < nsteps; ++t) {
     if (int rc = walk_launch(h)) return rc;
     h->pop = false;
@@ -500,11 +532,13 @@ int walk_steps(lbm_handle* h, int64_t nsteps) {
 }
 
 int run_moments(lbm_handle* h, double* rho, double* ux, double* uy) {
-  if (h->mom && rho && !ux && !uy) {
+  if (int rc = settle(h)) return rc;
+  const bool mom = h->mom && !h->graphs;
+  if (mom && rho && !ux && !uy) {
     LBM_CUDA(h, lbm::launch_density(h->p.precision, h->phys, h->m(h->mcur), h->Tf, rho, h->N, h->status, h->stream));
     return LBM_OK;
   }
-  if (h->mom) {
+  if (mom) {
     lbm::WalkIO io = walk_io(h, h->mcur);
     io.Tfield = h->Tf;
     io.rho_out = rho;
@@ -714,6 +748,7 @@ int lbm_init(const lbm_params* p, const double* rho0, int rho0_where, void* stre
   h->rho_mid = midpoint_level(h->p);
 
   e = cudaMemsetAsync(h->status, 0, sizeof(int), h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->pending(), 1, sizeof(int), h->stream);  // (not zero)
   if (e == cudaSuccess)
     e = lbm::launch_init(p->precision, rho_dev, h->f[0], p->nx, p->ny, rho_ref, h->parts[0], h->P, h->stream);
   if (e == cudaSuccess && p->thermal)
@@ -733,18 +768,21 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
   lbm::TraceRange trace("lbm_step");
   if (!h) { set_err(g_err, "handle is NULL"); return LBM_EINVAL; }
   if (nsteps < 0) { set_err(h->err, "nsteps must be >= 0"); return LBM_EINVAL; }
+  if (int rc = settle(h)) return rc;
   const bool block = nsteps + h->since_io >= kWalkSteps;  // not a single step between reads
   if (nsteps >= (h->p.precision == LBM_FP32 ? kColumnStepsF : kColumnStepsD) && h->tiling.variant == 0 &&
-      column_usable(h) && !(h->mom && capturing(h))) {
-    if (int rc = leave_moments(h)) return rc;
+      column_usable(h)) {
+    if (!h->graphs)
+      if (int rc = leave_moments(h)) return rc;
     h->parts_ok = false;
     h->since_io = kWalkSteps;
     LBM_CUDA(h, column_launch(h, h->f[h->cur], nsteps));
     h->steps += nsteps;
-    return LBM_OK;
+    return h->graphs ? refresh_partials(h) : LBM_OK;  // a graph's next call may be any
   }
-  if (walk_eligible(h) && (h->mom || (block && !capturing(h)))) return walk_steps(h, nsteps);
-  if (int rc = leave_moments(h)) return rc;
+  if (walk_eligible(h) && (h->mom || block)) return walk_steps(h, nsteps);
+  if (!h->graphs)
+    if (int rc = leave_moments(h)) return rc;
   if (int rc = ensure_partials(h)) return rc;
   h->since_io = int(std::min<int64_t>(h->since_io + nsteps, kWalkSteps));
   lbm::StepIO io{};
@@ -869,26 +907,29 @@ int lbm_set_state(lbm_handle* h, const double* f, int where, int64_t steps_done)
   lbm::TraceRange trace("lbm_set_state");
   if (!h) { set_err(g_err, "handle is NULL"); return LBM_EINVAL; }
   if (!f || (where != LBM_HOST && where != LBM_DEVICE)) { set_err(h->err, "bad f or where"); return LBM_EINVAL; }
-  h->pop = true;
-  h->mom = false;
-  h->since_io = 0;
+  // (the call waits for its copies, which no capture allows: a captured one is refused before the
+  // handle's own account of the state changes)
   if (where == LBM_DEVICE) {
     LBM_CUDA(h, lbm::launch_state_in(h->p.precision, f, h->f[h->cur], h->N, h->p.rho_ref, h->parts[h->pcur], h->P,
                                      h->stream));
-    h->npart = h->P;
-    h->parts_ok = true;
   } else {  // staged through ux, one plane at a time (stream-ordered)
     for (int i = 0; i < 9; ++i) {
       void* plane = static_cast<char*>(h->f[h->cur]) + size_t(i) * h->N * h->s;
       LBM_CUDA(h, cudaMemcpyAsync(h->ux, f + size_t(i) * h->N, h->N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
       LBM_CUDA(h, lbm::launch_plane_from_double(h->p.precision, h->ux, plane, h->N, kWeights[i] * h->p.rho_ref, h->stream));
     }
-    if (int rc = refresh_partials(h)) return rc;
+    LBM_CUDA(h, lbm::launch_partials(h->p.precision, h->f[h->cur], h->p.nx, h->p.ny, h->parts[h->pcur], h->P, h->stream));
   }
   LBM_CUDA(h, cudaMemsetAsync(h->status, 0, sizeof(int), h->stream));
+  if (h->graphs) LBM_CUDA(h, cudaMemsetAsync(h->pending(), 0, sizeof(int), h->stream));
+  LBM_CUDA(h, cudaStreamSynchronize(h->stream));
+  h->pop = true;
+  h->mom = false;
+  h->npart = h->P;
+  h->parts_ok = true;
+  h->since_io = 0;
   h->have_prev = false;
   h->steps = steps_done;
-  LBM_CUDA(h, cudaStreamSynchronize(h->stream));
   return LBM_OK;
 }
 

@@ -101,6 +101,7 @@ struct WalkIO {
   double *rho_out, *ux_out, *uy_out;  // moments: doubles [y][x] (may be NULL)
   void *rho_T, *ux_T, *uy_T;          // thermal step: this step's rho, u as reals [y][x]
   const void* Tfield;     // thermal: real[ny][nx] (NULL: uniform T)
+  const int* pending;     // populations: nothing is done where this device word is zero (NULL: always)
 };
 // the tiling of a lattice on a GPU of nsm SMs; at most max_ctas CTAs (partial sums), false where
 // that cannot be kept: such a tiling is not launched

@@ -156,6 +156,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? kWalkThreadsF : kWalkThreadsD
   const bool zh = tl.zh != 0;
   griddep_wait();  // launched as a dependent of the previous kernel: its state is complete
   griddep_launch_dependents();
+  if (MODE == WALK_POPULATIONS && io.pending && *io.pending == 0) return;
 
   struct Raw {
     L dr, jx, jy, t;
