@@ -121,6 +121,9 @@ cudaError_t launch_init(int precision, const double* rho0, void* f, int nx, int 
                         int npart, cudaStream_t stream);
 cudaError_t launch_partials(int precision, const void* f, int nx, int ny, double* part, int npart,
                             cudaStream_t stream);
+// the same of one plane of nx ny values
+cudaError_t launch_plane_partials(int precision, const void* plane, int nx, int ny, double* part, int npart,
+                                  cudaStream_t stream);
 // out[0] = sum of part[0..npart) in a fixed order
 cudaError_t launch_sum_partials(const double* part, int npart, double* out, cudaStream_t stream);
 // one population plane of n values: out = plane + add / plane = in - sub

@@ -792,10 +792,11 @@ __global__ void init_kernel(const double* __restrict__ rho0, T* __restrict__ f, 
   block_partial(acc, part);
 }
 
-// ---- FP64 partial sums of sum_i g_i: block b covers vector groups [b*chunk, (b+1)*chunk).
+// ---- FP64 partial sums of sum_i g_i over PLANES planes (9: a state's populations, 1: the density of
+// one held as moments): block b covers vector groups [b*chunk, (b+1)*chunk).
 // FP32 storage: every value into the per-thread two-sum pairs (GB300's FP64 pipe is slow),
 // four nodes a thread per plane; FP64 storage: plain FP64 sums, two nodes a thread.
-template <typename T>
+template <typename T, int PLANES>
 __global__ void partials_kernel(const T* __restrict__ f, int nx, int ny, double* __restrict__ part) {
   using Q = Quad<T>;
   using V = typename Q::V;
@@ -806,11 +807,11 @@ __global__ void partials_kernel(const T* __restrict__ f, int nx, int ny, double*
   Acc<V> acc;
 #pragma unroll 2
   for (size_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
-    V g[9][2];
+    V g[PLANES][2];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) Q::load(f + i * n + k * NQ, g[i]);
+    for (int i = 0; i < PLANES; ++i) Q::load(f + i * n + k * NQ, g[i]);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
+    for (int i = 0; i < PLANES; ++i) {
       acc.add(g[i][0], i % 3);
       acc.add(g[i][1], i % 3);
     }
@@ -1218,9 +1219,17 @@ cudaError_t launch_init(int precision, const double* rho0, void* f, int nx, int 
 cudaError_t launch_partials(int precision, const void* f, int nx, int ny, double* part, int npart,
                             cudaStream_t stream) {
   if (precision == 1)
-    partials_kernel<float><<<npart, 256, 0, stream>>>(static_cast<const float*>(f), nx, ny, part);
+    partials_kernel<float, 9><<<npart, 256, 0, stream>>>(static_cast<const float*>(f), nx, ny, part);
   else
-    partials_kernel<double><<<npart, 256, 0, stream>>>(static_cast<const double*>(f), nx, ny, part);
+    partials_kernel<double, 9><<<npart, 256, 0, stream>>>(static_cast<const double*>(f), nx, ny, part);
+  return cudaGetLastError();
+}
+cudaError_t launch_plane_partials(int precision, const void* plane, int nx, int ny, double* part, int npart,
+                                  cudaStream_t stream) {
+  if (precision == 1)
+    partials_kernel<float, 1><<<npart, 256, 0, stream>>>(static_cast<const float*>(plane), nx, ny, part);
+  else
+    partials_kernel<double, 1><<<npart, 256, 0, stream>>>(static_cast<const double*>(plane), nx, ny, part);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,61 @@
+"""When a handle changes between its two forms, populations and moments: what a call takes shows in the
+last bits of its result (the two steps round differently), so the routes are compared bit by bit.
+"""
+import numpy as np
+import pytest
+
+from paper_2301_12869_gb300 import lbm
+from test_gpu_walk import cuda_lib, read, setup  # noqa: F401 (the fixture is used)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("nx, ny, precision, zh", [(256, 200, "fp32", False), (256, 200, "fp32", True),
+                                                   (256, 257, "fp64", False)])
+def test_single_steps_between_reads_are_population_steps(nx, ny, precision, zh):
+    """After a block of steps on moments, a loop of one step and a read of the populations takes one
+    population step a turn, not a walk and a collision that forms the populations again."""
+    p, _, rho0, f = setup(nx, ny, precision, 2, zh)
+    out = []
+    for populations in (False, True):
+        h = lbm.lbm_init(p, rho0)
+        try:
+            lbm.lbm_set_state(h, f)
+            lbm.lbm_step(h, 9)
+            states = [read(h, p)]
+            if populations:
+                lbm.lbm_set_tiling(h, 0)  # the state as populations, as lbm_set_tiling leaves it
+            for _ in range(3):
+                lbm.lbm_step(h, 1)
+                states.append(read(h, p))
+            out.append(states)
+        finally:
+            lbm.lbm_destroy(h)
+    for k, (a, b) in enumerate(zip(*out)):
+        assert np.array_equal(a, b), k
+
+
+@pytest.mark.parametrize("form", [1, 2])
+@pytest.mark.parametrize("zh", [False, True])
+def test_mass_of_a_state_on_moments(form, zh):
+    """The collision keeps a node's mass, so the mass of the populations after n steps is the sum of the
+    densities they collided from: taken from there without forming the populations, it is that sum to
+    1e-13 (sums of the rounded FP32 populations differ from it by 1e-11)."""
+    nx, ny = 256, 200
+    p, _, rho0, f = setup(nx, ny, "fp32", form, zh)
+    h = lbm.lbm_init(p, rho0)
+    try:
+        lbm.lbm_set_state(h, f)
+        lbm.lbm_step(h, 8)
+        rho = np.empty((ny, nx))
+        for _ in range(2):
+            lbm.lbm_moments(h, rho)
+            lbm.lbm_step(h, 1)
+            assert lbm.lbm_reduce(h, lbm.LBM_REDUCE_MASS)[0] == pytest.approx(float(np.sum(rho)), rel=1e-13)
+            assert lbm.lbm_reduce(h, lbm.LBM_REDUCE_MEAN_RHO)[0] == pytest.approx(float(np.mean(rho)), rel=1e-13)
+        mass = lbm.lbm_reduce(h, lbm.LBM_REDUCE_MASS)[0]
+        got = read(h, p)
+        assert mass == pytest.approx(float(np.sum(got)), rel=1e-9)
+        assert lbm.lbm_reduce(h, lbm.LBM_REDUCE_MASS)[0] == pytest.approx(float(np.sum(got)), rel=1e-13)
+    finally:
+        lbm.lbm_destroy(h)
