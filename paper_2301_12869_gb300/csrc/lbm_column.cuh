@@ -33,6 +33,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <cfloat>
 #include <cmath>
 #include <cstdint>
 
@@ -44,7 +45,7 @@ template <>
 struct ItemOf<float> {
   using V = f2;
   using S = dd;  // sums of drho
-  using M = float;  // largest change
+  using M = dd;  // largest change
   static constexpr int N = 2, Q = 4, max_threads = 256;
 };
 template <>
@@ -58,7 +59,7 @@ template <>
 struct ItemOf<dd> {
   using V = dd;
   using S = dd;
-  using M = float;
+  using M = dd;
   static constexpr int N = 1, Q = 1, max_threads = 256;
 };
 
@@ -176,24 +177,37 @@ __device__ __forceinline__ Lane<V, N> two_sum_error(const Lane<V, N>& a, const L
   return (a - (s - bb)) + (b - bb);
 }
 
-// largest |rho - previous rho| of an item from (value, low part) pairs: exact to FP32 relative
-// (the FP64 pipe is left to FP64 columns)
-__device__ __forceinline__ float item_change(const Lane<f2, 2>& a, const Lane<f2, 2>& al, const Lane<f2, 2>& b,
-                                              const Lane<f2, 2>& bl) {
-  const Lane<f2, 2> d = (a - b) + (al - bl);
-  float m = 0.f;  // a NaN does not count
+// the larger of m and d; a NaN d does not count
+__device__ __forceinline__ dd larger(dd m, dd d) { return d.hi > m.hi || (d.hi == m.hi && d.lo > m.lo) ? d : m; }
+__device__ __forceinline__ double larger(double m, double d) { return fmax(m, d); }
+__device__ __forceinline__ dd magnitude(dd d) { return d.hi < 0.f ? -d : d; }
+// |(a + al) - (b + bl)|: the difference of the values is exact, so the pair is good to 2^-24 of the
+// change beyond what the low parts hold
+__device__ __forceinline__ dd change(float a, float al, float b, float bl) {
+  const dd s = dd_two_sum(a, -b);
+  if (!(fabsf(s.hi) <= FLT_MAX)) return dd{fabsf(s.hi), 0.f};  // infinite: no error terms
+  return magnitude(dd_two_sum(s.hi, __fadd_rn(s.lo, __fsub_rn(al, bl))));
+}
+
+// largest |rho - previous rho| of an item from (value, low part) pairs, as a pair: it decides
+// convergence and is the caller's residual in FP64 (the FP64 pipe is left to FP64 columns)
+__device__ __forceinline__ dd item_change(const Lane<f2, 2>& a, const Lane<f2, 2>& al, const Lane<f2, 2>& b,
+                                          const Lane<f2, 2>& bl) {
+  dd m{};
 #pragma unroll
-  for (int j = 0; j < 2; ++j) m = fmaxf(m, fmaxf(fabsf(lo(d.v[j])), fabsf(hi(d.v[j]))));
+  for (int j = 0; j < 2; ++j) {
+    m = larger(m, change(lo(a.v[j]), lo(al.v[j]), lo(b.v[j]), lo(bl.v[j])));
+    m = larger(m, change(hi(a.v[j]), hi(al.v[j]), hi(b.v[j]), hi(bl.v[j])));
+  }
   return m;
 }
 __device__ __forceinline__ double item_change(const Lane<double, 1>& a, const Lane<double, 1>&,
                                               const Lane<double, 1>& b, const Lane<double, 1>&) {
   return fmax(0.0, fabs(a.v[0] - b.v[0]));
 }
-__device__ __forceinline__ float item_change(const Lane<dd, 1>& a, const Lane<dd, 1>&, const Lane<dd, 1>& b,
-                                             const Lane<dd, 1>&) {
-  const dd d = a.v[0] - b.v[0];
-  return fmaxf(0.f, fabsf(__fadd_rn(d.hi, d.lo)));
+__device__ __forceinline__ dd item_change(const Lane<dd, 1>& a, const Lane<dd, 1>&, const Lane<dd, 1>& b,
+                                          const Lane<dd, 1>&) {
+  return larger(dd{}, change(a.v[0].hi, a.v[0].lo, b.v[0].hi, b.v[0].lo));
 }
 
 // pull streaming (Eq. LBE) of node (x, y): the nine populations arriving there
@@ -517,23 +531,23 @@ __global__ void __launch_bounds__(ItemOf<T>::max_threads, sizeof(T) == 4 && R > 
           }
       }
       if (chk) {  // max |rho_t - rho_(t-1)| over the column
-        M rm = 0;
+        M rm{};
 #pragma unroll
         for (int q = 0; q < R; ++q)
           if (live(q)) {
             const L pl = LOW ? load_item(prev + NN + node(q)) : zeroL;
-            rm = max(rm, item_change(dr[q], dl[q], load_item(prev + node(q)), pl));
+            rm = larger(rm, item_change(dr[q], dl[q], load_item(prev + node(q)), pl));
           }
 #pragma unroll
-        for (int mm = 16; mm; mm >>= 1) rm = max(rm, __shfl_xor_sync(0xffffffffu, rm, mm));
+        for (int mm = 16; mm; mm >>= 1) rm = larger(rm, lane_value(rm, lane ^ mm));
         if (lane < cs) {
           M* dst = &max_s[rank * NW + warp];
           *(cs > 1 ? cluster.map_shared_rank(dst, lane) : dst) = rm;
         }
         sync();
-        M rmax = 0;
-        for (int q = 0; q < cs * NW; ++q) rmax = max(rmax, max_s[q]);
-        const double r = double(rmax);
+        M rmax{};
+        for (int q = 0; q < cs * NW; ++q) rmax = larger(rmax, max_s[q]);
+        const double r = hsum(rmax);
         res = r;
         if (!(r > run.tol)) {  // converged (uniform)
           last = true;
