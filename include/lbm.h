@@ -266,8 +266,7 @@ int lbm_batch_run_stall(lbm_batch* b, double tol, int64_t max_steps, int check_e
  * captures the damped oscillations in which the columns' slow modes decay. The estimate
  * replaces the state when every density stays positive, and is undone when the next
  * residual check is worse than the one before it (x: the populations, or with every
- * relaxation time 1 the moments rho, j of the streamed ones, which determine them; no estimate
- * is taken at a run's last step). checks = 0 turns it off. The library
+ * relaxation time 1 the moments rho, j of the streamed ones, which determine them). checks = 0 turns it off. The library
  * allocates 6 x 9 x (total nodes) reals once. Not carried over by lbm_batch_convert. */
 int lbm_batch_set_acceleration(lbm_batch* b, int checks);
 

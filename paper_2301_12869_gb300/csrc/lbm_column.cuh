@@ -549,13 +549,141 @@ __global__ void __launch_bounds__(ItemOf<T>::max_threads, sizeof(T) == 4 && R > 
         for (int q = 0; q < cs * NW; ++q) rmax = larger(rmax, max_s[q]);
         const double r = hsum(rmax);
         res = r;
+        bool stop = false;
         if (!(r > run.tol)) {  // converged (uniform)
-          last = true;
+          last = stop = true;
         } else if (r < 0.99 * best) {
           best = r;
           stalled = 0;
         } else if (run.stall_checks > 0 && r < kStallBelow<T> && ++stalled >= run.stall_checks) {
-          last = true;  // no gain near the precision's rounding floor
+          last = stop = true;  // no gain near the precision's rounding floor
+        }
+        if (ACC && mpe && !stop) {
+          // ---- minimal polynomial extrapolation on the moments (see lbm_batch.cu), ahead of their
+          // collision, so that a run's last step takes part too: its populations are the collision of
+          // the estimate
+          auto keep = [&](T* dst) {
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+              if (live(q)) {
+                store_item(dst + node(q), dr[q]);
+                store_item(dst + NN + node(q), jx[q]);
+                store_item(dst + 2 * NN + node(q), jy[q]);
+              }
+          };
+          auto take = [&](const T* src) {
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+              if (live(q)) {
+                dr[q] = load_item(src + node(q));
+                jx[q] = load_item(src + NN + node(q));
+                jy[q] = load_item(src + 2 * NN + node(q));
+                dl[q] = zeroL;
+              }
+          };
+          auto remass = [&] {
+            if (mean) {
+              sync();
+              moments_mass();
+            }
+          };
+          if (verify) {
+            // the first check after an extrapolation: a larger change than before it means the
+            // estimate is worse - back to the last snapshot
+            verify = false;
+            if (res > res_before) {
+              take(slot(kMpeK + 1));
+              remass();
+              skip_cycle = true;
+              nsnap = 0;
+              checks_since = 0;
+            }
+          }
+          if (++checks_since >= run.mpe_checks) {
+            checks_since = 0;
+            keep(slot(nsnap));
+            if (++nsnap == kMpeK + 2) {
+              nsnap = 0;
+              if (skip_cycle) {
+                skip_cycle = false;
+              } else {
+                double G[NG];
+#pragma unroll
+                for (int i = 0; i < NG; ++i) G[i] = 0.0;
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                  if (!live(q)) continue;
+                  for (int e = 0; e < 3 * Q; ++e) {  // component e / Q, node e % Q
+                    const size_t at = size_t(e / Q) * NN + node(q) + size_t(e % Q);
+                    double x[NU + 1];
+#pragma unroll
+                    for (int j = 0; j <= NU; ++j) x[j] = hsum(slot(j)[at]);
+                    int p = 0;
+#pragma unroll
+                    for (int i = 0; i < NU; ++i)
+#pragma unroll
+                      for (int j = i; j < NU; ++j) G[p++] += (x[i + 1] - x[i]) * (x[j + 1] - x[j]);
+                  }
+                }
+#pragma unroll
+                for (int i = 0; i < NG; ++i) {
+                  const double v = lanes_total(G[i], 32);
+                  if (lane == 0) *(cs > 1 ? cluster.map_shared_rank(&gram_s[i][rank * NW + warp], 0) : &gram_s[i][warp]) = v;
+                }
+                sync();
+                if (rank == 0 && tid == 0) {
+                  double g[NG], gam[NU];
+                  for (int i = 0; i < NG; ++i) {
+                    g[i] = 0.0;
+                    for (int w = 0; w < cs * NW; ++w) g[i] += gram_s[i][w];
+                  }
+                  const bool ok = mpe_solve(g, gam);
+                  for (int r = 0; r < cs; ++r) {
+                    double* dst = cs > 1 ? cluster.map_shared_rank(gam_s, r) : gam_s;
+                    for (int j = 0; j < NU; ++j) dst[j] = gam[j];
+                    *(cs > 1 ? cluster.map_shared_rank(&ok_s, r) : &ok_s) = ok ? 1 : 0;
+                  }
+                }
+                sync();
+                if (ok_s) {
+                  double gam[NU];
+                  for (int j = 0; j < NU; ++j) gam[j] = gam_s[j];
+                  int bad = 0;
+#pragma unroll
+                  for (int q = 0; q < R; ++q) {
+                    if (!live(q)) continue;
+                    for (int e = 0; e < 3 * Q; ++e) {
+                      const size_t at = size_t(e / Q) * NN + node(q) + size_t(e % Q);
+                      double acc = 0.0;
+                      for (int j = 0; j < NU; ++j) acc += gam[j] * hsum(slot(j)[at]);
+                      if (e < Q) {
+                        if (!(col.rho_ref + acc > 0.0)) bad = 1;
+                        set_node(dr[q], e, acc);
+                      } else if (e < 2 * Q) {
+                        set_node(jx[q], e - Q, acc);
+                      } else {
+                        set_node(jy[q], e - 2 * Q, acc);
+                      }
+                    }
+                    dl[q] = zeroL;
+                  }
+                  bad = __syncthreads_or(bad);
+                  if (cs > 1) {
+                    if (tid < cs) *cluster.map_shared_rank(&bad_s[rank], tid) = bad;
+                    sync();
+                    for (int r = 0; r < cs; ++r) bad |= bad_s[r];
+                  }
+                  if (bad)
+                    take(slot(kMpeK + 1));  // the state before
+                  remass();
+                  if (!bad) {
+                    verify = true;
+                    res_before = res;
+                  }
+                }
+              }
+            }
+          }
         }
       }
       // ---- psi and its stencil sums
@@ -708,132 +836,6 @@ __global__ void __launch_bounds__(ItemOf<T>::max_threads, sizeof(T) == 4 && R > 
         zmean = mc;
       }
       if (mean) moments_mass();
-
-      if (ACC && mpe && chk) {
-        // ---- minimal polynomial extrapolation on the moments (see lbm_batch.cu)
-        auto keep = [&](T* dst) {
-#pragma unroll
-          for (int q = 0; q < R; ++q)
-            if (live(q)) {
-              store_item(dst + node(q), dr[q]);
-              store_item(dst + NN + node(q), jx[q]);
-              store_item(dst + 2 * NN + node(q), jy[q]);
-            }
-        };
-        auto take = [&](const T* src) {
-#pragma unroll
-          for (int q = 0; q < R; ++q)
-            if (live(q)) {
-              dr[q] = load_item(src + node(q));
-              jx[q] = load_item(src + NN + node(q));
-              jy[q] = load_item(src + 2 * NN + node(q));
-              dl[q] = zeroL;
-            }
-        };
-        auto remass = [&] {
-          if (mean) {
-            sync();
-            moments_mass();
-          }
-        };
-        if (verify) {
-          // the first check after an extrapolation: a larger change than before it means the
-          // estimate is worse - back to the last snapshot
-          verify = false;
-          if (res > res_before) {
-            take(slot(kMpeK + 1));
-            remass();
-            skip_cycle = true;
-            nsnap = 0;
-            checks_since = 0;
-          }
-        }
-        if (++checks_since >= run.mpe_checks) {
-          checks_since = 0;
-          keep(slot(nsnap));
-          if (++nsnap == kMpeK + 2) {
-            nsnap = 0;
-            if (skip_cycle) {
-              skip_cycle = false;
-            } else {
-              double G[NG];
-#pragma unroll
-              for (int i = 0; i < NG; ++i) G[i] = 0.0;
-#pragma unroll
-              for (int q = 0; q < R; ++q) {
-                if (!live(q)) continue;
-                for (int e = 0; e < 3 * Q; ++e) {  // component e / Q, node e % Q
-                  const size_t at = size_t(e / Q) * NN + node(q) + size_t(e % Q);
-                  double x[NU + 1];
-#pragma unroll
-                  for (int j = 0; j <= NU; ++j) x[j] = hsum(slot(j)[at]);
-                  int p = 0;
-#pragma unroll
-                  for (int i = 0; i < NU; ++i)
-#pragma unroll
-                    for (int j = i; j < NU; ++j) G[p++] += (x[i + 1] - x[i]) * (x[j + 1] - x[j]);
-                }
-              }
-#pragma unroll
-              for (int i = 0; i < NG; ++i) {
-                const double v = lanes_total(G[i], 32);
-                if (lane == 0) *(cs > 1 ? cluster.map_shared_rank(&gram_s[i][rank * NW + warp], 0) : &gram_s[i][warp]) = v;
-              }
-              sync();
-              if (rank == 0 && tid == 0) {
-                double g[NG], gam[NU];
-                for (int i = 0; i < NG; ++i) {
-                  g[i] = 0.0;
-                  for (int w = 0; w < cs * NW; ++w) g[i] += gram_s[i][w];
-                }
-                const bool ok = mpe_solve(g, gam);
-                for (int r = 0; r < cs; ++r) {
-                  double* dst = cs > 1 ? cluster.map_shared_rank(gam_s, r) : gam_s;
-                  for (int j = 0; j < NU; ++j) dst[j] = gam[j];
-                  *(cs > 1 ? cluster.map_shared_rank(&ok_s, r) : &ok_s) = ok ? 1 : 0;
-                }
-              }
-              sync();
-              if (ok_s) {
-                double gam[NU];
-                for (int j = 0; j < NU; ++j) gam[j] = gam_s[j];
-                int bad = 0;
-#pragma unroll
-                for (int q = 0; q < R; ++q) {
-                  if (!live(q)) continue;
-                  for (int e = 0; e < 3 * Q; ++e) {
-                    const size_t at = size_t(e / Q) * NN + node(q) + size_t(e % Q);
-                    double acc = 0.0;
-                    for (int j = 0; j < NU; ++j) acc += gam[j] * hsum(slot(j)[at]);
-                    if (e < Q) {
-                      if (!(col.rho_ref + acc > 0.0)) bad = 1;
-                      set_node(dr[q], e, acc);
-                    } else if (e < 2 * Q) {
-                      set_node(jx[q], e - Q, acc);
-                    } else {
-                      set_node(jy[q], e - 2 * Q, acc);
-                    }
-                  }
-                  dl[q] = zeroL;
-                }
-                bad = __syncthreads_or(bad);
-                if (cs > 1) {
-                  if (tid < cs) *cluster.map_shared_rank(&bad_s[rank], tid) = bad;
-                  sync();
-                  for (int r = 0; r < cs; ++r) bad |= bad_s[r];
-                }
-                if (bad)
-                  take(slot(kMpeK + 1));  // the state before
-                remass();
-                if (!bad) {
-                  verify = true;
-                  res_before = res;
-                }
-              }
-            }
-          }
-        }
-      }
     }
     const int any = __syncthreads_or(flag);
     if (tid == 0 && any) {

@@ -1,9 +1,11 @@
 """What columns on chip do at a residual check: the residual itself, formed in FP64 from the library's
-own states."""
+own states, and one extrapolation cycle, formed in FP64 from the library's own snapshots."""
+import numpy as np
 import pytest
 
 from oracle import lbm as olbm
-from test_gpu_column import cuda_lib, run  # noqa: F401 (the fixture is used)
+from paper_2301_12869_gb300 import lbm
+from test_gpu_column import A, T_C, columns, cuda_lib, run, split  # noqa: F401 (the fixture is used)
 
 pytestmark = pytest.mark.gpu
 
@@ -24,3 +26,57 @@ def test_residual_beyond_the_storage_type(precision, zh, steps):
     for f0, f1, op, r in zip(*states, ops, res):
         want = olbm.residual(olbm.macroscopic(f1, op).rho, olbm.macroscopic(f0, op).rho)
         assert abs(r - want) <= tol, (op.ny, r, want)
+
+
+def moments(f):
+    g = olbm.stream(f)
+    return np.stack([g.sum(axis=0), np.tensordot(olbm.C[:, 0], g, 1), np.tensordot(olbm.C[:, 1], g, 1)])
+
+
+def extrapolated(states):
+    """Minimal polynomial extrapolation of order 4 of six states: their weights, which are those of
+    the moments' differences."""
+    x = [moments(f).ravel() for f in states]
+    u = np.stack([x[j + 1] - x[j] for j in range(5)], axis=1)
+    c = np.append(np.linalg.lstsq(u[:, :4], -u[:, 4], rcond=None)[0], 1.0)
+    return c / c.sum()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "dd", "fp64"])
+def test_one_extrapolation_cycle(precision):
+    """A run of one cycle (six snapshots, one every two checks) ends with the step from the
+    estimate, like a run whose cycle ends before its last step. The populations are then the collision of
+    the snapshots' weighted mean. Rounding the snapshots' moments (1e-8, 1e-15) moves the estimate by 2e-6
+    (FP32) and 3e-13 (double-float) of its distance from the plain state here, storing it by 3e-6 and 3e-13."""
+    nx, heights, every, checks = 4, (40, 64, 300), 25, 2
+    cols, rhos = columns(nx, heights)
+    flat = np.concatenate([r.ravel() for r in rhos])
+    p = lbm.make_params(nx, 8, 0.8 * T_C, precision, a=A)
+    n = 9 * nx * sum(heights)
+
+    def states(steps, acc):
+        b = lbm.lbm_batch_init(p, cols, flat)
+        try:
+            if acc:
+                lbm.lbm_batch_set_acceleration(b, checks)
+            lbm.lbm_batch_run(b, 0.0, steps, every)
+            f = np.empty(n)
+            lbm.lbm_batch_get_state(b, f)
+            return split(f, nx, heights)
+        finally:
+            lbm.lbm_batch_destroy(b)
+
+    last = 6 * checks * every
+    plain = [states(k * checks * every - 1, False) for k in range(1, 7)]  # what the snapshots' steps start from
+    got, without = states(last, True), states(last, False)
+    ops = [olbm.Params(nx=nx, ny=c["ny"], a=A, T=c["T"], g=(c["gx"], c["gy"]), form=c["form"]) for c in cols]
+    for j, op in enumerate(ops):
+        w = extrapolated([s[j] for s in plain])
+        want = olbm.step(sum(wk * s[j] for wk, s in zip(w, plain[:5])), op)
+        moved = float(np.max(np.abs(want - without[j])))
+        err = float(np.max(np.abs(got[j] - want)))
+        assert moved > 1e-4 and err <= TOLERANCE[precision] * moved, (op.ny, err, moved)
+
+
+# of that distance
+TOLERANCE = {"fp32": 1e-4, "dd": 1e-10, "fp64": 1e-11}
