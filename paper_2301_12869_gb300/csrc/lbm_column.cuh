@@ -12,7 +12,7 @@
 // FP64 or double-float node, whose arithmetic is the bound and wants the most warps), up to R
 // such items; a row takes 2^row_log2 lanes of a warp, so x neighbours (periodic) come by
 // shuffles. y neighbours go through shared memory, once for the potential's stencil sums
-//   A = psi_x difference / 12, B = psi/3 + (psi(x-1) + psi(x+1))/12
+//   A = psi_x difference / 12, B = psi/3 + (psi(x-1) + psi(x+1))/12  (double-float: 3 sqrt(3) times)
 //   S_x = 4 A(y) + A(y+1) + A(y-1),  S_y = B(y+1) - B(y-1)
 // and once for what a node sends up (u1 = f2 + f5(x-1) + f6(x+1), u2 = f5(x-1) - f6(x+1)) and
 // down (v1, v2 of f4, f8, f7). Two barriers a step; a cluster's CTAs write their edge rows into
@@ -78,22 +78,33 @@ __device__ __forceinline__ double real<double>(double c) { return c; }
 template <>
 __device__ __forceinline__ dd real<dd>(double c) { return dd_of(c); }
 
+// Double-float columns hold sqrt(3) psi, and its stencil sums without their factor 1/3: psi^2 then has
+// no constant that is a third (3 k_2, 3 k_3 are exact for the usual a, G), and the force takes -G/9 and
+// the sigma term 1/27. The double-float 1/3 is 2^-50 too small at every step alike: over 300 steps of
+// 384 columns of 64 rows the populations' error against FP64 was 5.1e-14 with it, and is 3.0e-14 (4.3e-14
+// in the order of lbm_physics.cuh, which has it too but rounds differently); two products a node less.
+template <typename V>
+constexpr double kPsi2 = 1.0;  // the square of the factor
+template <>
+constexpr double kPsi2<dd> = 3.0;
+
 template <typename V>
 __device__ UnitT<V> column_unit(const ColumnArgs& a, const BatchCol& c) {
+  constexpr double s = kPsi2<V>;
   UnitT<V> u{};
   u.p.rho_ref = real<V>(c.rho_ref);
   u.p.RT = real<V>(c.RT);
   u.p.a = real<V>(a.a);
   u.p.b4 = real<V>(a.b / 4.0);
   u.p.twoOverG = real<V>(2.0 / a.G);
-  u.p.negG = real<V>(-a.G);
+  u.p.negG = real<V>(-a.G / (s * s));
   u.p.gx = real<V>(c.gx);
   u.p.gy = real<V>(c.gy);
   u.p.form = c.form;
-  u.k1 = real<V>(2.0 * c.RT / a.G);
-  u.p.k2 = real<V>(-2.0 * a.a / a.G);
-  u.p.k3 = real<V>(-2.0 / (3.0 * a.G));
-  u.p.kS = real<V>(a.G * a.G * a.sig_e / 72.0);
+  u.k1 = real<V>(2.0 * s * c.RT / a.G);
+  u.p.k2 = real<V>(-2.0 * s * a.a / a.G);
+  u.p.k3 = real<V>(s == 3.0 ? -2.0 / a.G : -2.0 / (3.0 * a.G));
+  u.p.kS = real<V>(a.G * a.G * a.sig_e / (72.0 * s * s * s));
   return u;
 }
 
@@ -700,10 +711,17 @@ __global__ void __launch_bounds__(ItemOf<T>::max_threads, sizeof(T) == 4 && R > 
           if (live(q)) flag |= fl;
         }
         const L w = left(psi[q]), e = right(psi[q]);
-        const L A = cst<V>(1.0 / 12.0) * (e - w);
-        L B;
+        L A = e - w, B;
 #pragma unroll
-        for (int j = 0; j < N; ++j) B.v[j] = cst<V>(1.0 / 3.0) * fma2(0.25, e.v[j] + w.v[j], psi[q].v[j]);
+        for (int j = 0; j < N; ++j) {
+          B.v[j] = fma2(0.25, e.v[j] + w.v[j], psi[q].v[j]);
+          if constexpr (kPsi2<V> == 3.0) {
+            A.v[j] = scale2(0.25, A.v[j]);
+          } else {
+            A.v[j] = cst<V>(1.0 / 12.0) * A.v[j];
+            B.v[j] = cst<V>(1.0 / 3.0) * B.v[j];
+          }
+        }
         if (live(q)) {
           sA[s] = A;
           sB[s] = B;

@@ -3,8 +3,9 @@ own states, and one extrapolation cycle, formed in FP64 from the library's own s
 import numpy as np
 import pytest
 
+from oracle import eos
 from oracle import lbm as olbm
-from paper_2301_12869_gb300 import lbm
+from paper_2301_12869_gb300 import inputs, lbm
 from test_gpu_column import A, T_C, columns, cuda_lib, run, split  # noqa: F401 (the fixture is used)
 
 pytestmark = pytest.mark.gpu
@@ -80,3 +81,28 @@ def test_one_extrapolation_cycle(precision):
 
 # of that distance
 TOLERANCE = {"fp32": 1e-4, "dd": 1e-10, "fp64": 1e-11}
+
+
+def test_double_float_error_over_a_block_of_steps():
+    """32 columns of 64 rows, 300 steps, against FP64: 3.0e-14 of the populations' norm in a numpy
+    emulation of the kernel's arithmetic over 384 such columns, 4.3e-14 in that of the general kernel and
+    5.1e-14 with a constant 1/3 in psi and its stencil; 32 columns spread by 5 %."""
+    ncol, nx, ny, steps = 32, 4, 64, 300
+    rng = np.random.default_rng(1)
+    T, gy = rng.uniform(0.75, 0.9, ncol) * T_C, -(10 ** rng.uniform(-5.5, -4.3, ncol))
+    cols, rhos = [], []
+    for k in range(ncol):
+        rv, rl, _ = eos.maxwell(T[k], A, 4.0, 1.0)
+        cols.append(dict(ny=ny, T=float(T[k]), gx=0.0, gy=float(gy[k]), form=1 + k % 2))
+        rhos.append(inputs.column_rho0(nx, ny, rl, rv, ny // 2, width=4.0))
+    b = lbm.lbm_batch_init(lbm.make_params(nx, 8, 0.8 * T_C, "dd", a=A), cols, np.concatenate([r.ravel() for r in rhos]))
+    try:
+        lbm.lbm_batch_run(b, 0.0, steps, 1000)
+        f = np.empty(9 * nx * ny * ncol)
+        lbm.lbm_batch_get_state(b, f)
+    finally:
+        lbm.lbm_batch_destroy(b)
+    want = np.stack([olbm.run(olbm.init_state(r), olbm.Params(nx=nx, ny=ny, a=A, T=c["T"], g=(0.0, c["gy"]), form=c["form"]),
+                              steps) for r, c in zip(rhos, cols)])
+    got = np.stack(split(f, nx, [ny] * ncol))
+    assert np.linalg.norm(got - want) / np.linalg.norm(want) <= 4.0e-14
