@@ -279,7 +279,9 @@ int lbm_batch_set_threads(lbm_batch* b, int threads);
  * every column runs `steps` (>= 1) steps with no residual stop (after a 2-step warm-up) for
  * each candidate block size, timed with CUDA events on the batch's stream; the fastest is
  * kept (lbm_batch_set_threads). threads[3] and us[3] (host, may be NULL) receive the
- * candidates and their microseconds per step of the whole batch. The batch's own state,
+ * candidates and their microseconds per step of the whole batch. Columns iterated on chip are
+ * measured once, which stands for all three: the block size stays what it is, the first
+ * candidate listed. The batch's own state,
  * step counts and residuals are not touched; the copy needs as much device memory as the
  * batch. Synchronises. */
 int lbm_batch_autotune(lbm_batch* b, int steps, int* threads, double* us);

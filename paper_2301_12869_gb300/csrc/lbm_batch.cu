@@ -1020,8 +1020,13 @@ int lbm_batch_autotune(lbm_batch* b, int steps, int* threads, double* us) {
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
   double best_us = 0.0;
   int best = b->threads;
-  for (int i = 0; i < 3 && e == cudaSuccess; ++i) {
-    t->threads = kThreadChoices[i];
+  // columns on chip have no block size to choose: one measurement, the present choice first and kept
+  const bool on_chip = !b->classes.empty();
+  int choices[3];
+  std::copy(std::begin(kThreadChoices), std::end(kThreadChoices), choices);
+  if (on_chip) std::rotate(choices, std::find(choices, choices + 3, best), choices + 3);
+  for (int i = 0; i < (on_chip ? 1 : 3) && e == cudaSuccess; ++i) {
+    t->threads = choices[i];
     size_grids(t);
     float ms = 0.f;
     // every column `steps` steps (tol < 0: no column stops early), after a 2-step warm-up
@@ -1036,11 +1041,13 @@ int lbm_batch_autotune(lbm_batch* b, int steps, int* threads, double* us) {
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
     if (e != cudaSuccess) break;
     const double v = 1e3 * double(ms) / steps;
-    if (threads) threads[i] = kThreadChoices[i];
-    if (us) us[i] = v;
+    for (int k = i; k < (on_chip ? 3 : i + 1); ++k) {
+      if (threads) threads[k] = choices[k];
+      if (us) us[k] = v;
+    }
     if (i == 0 || v < best_us) {
       best_us = v;
-      best = kThreadChoices[i];
+      best = choices[i];
     }
   }
   if (e0) cudaEventDestroy(e0);
@@ -1063,7 +1070,8 @@ int lbm_batch_run_stall(lbm_batch* b, double tol, int64_t max_steps, int check_e
   RunParams rp{tol, (long long)max_steps, check_every, stall_checks, b->snap ? b->mpe_checks : 0, b->snap,
                9 * b->total_nodes};
   cudaError_t e = cudaMemcpyAsync(b->run_d, &rp, sizeof(rp), cudaMemcpyHostToDevice, b->stream);
-  if (e == cudaSuccess && b->graph && (b->graph_acc != accelerated(b) || b->graph_threads != b->threads)) {
+  const bool sized = b->classes.empty();  // the block size is a choice
+  if (e == cudaSuccess && b->graph && (b->graph_acc != accelerated(b) || (sized && b->graph_threads != b->threads))) {
     // the kernel choice changed
     cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;

@@ -106,3 +106,17 @@ def test_double_float_error_over_a_block_of_steps():
                               steps) for r, c in zip(rhos, cols)])
     got = np.stack(split(f, nx, [ny] * ncol))
     assert np.linalg.norm(got - want) / np.linalg.norm(want) <= 4.0e-14
+
+
+def test_block_size_of_columns_on_chip():
+    """Their block size follows their height: nothing to choose, so one measurement stands for the
+    three candidates, and what lbm_batch_set_threads set stays."""
+    cols, rhos = columns(4, (40, 64))
+    b = lbm.lbm_batch_init(lbm.make_params(4, 8, 0.8 * T_C, "fp32", a=A), cols, np.concatenate([r.ravel() for r in rhos]))
+    try:
+        lbm.lbm_batch_set_threads(b, 512)
+        kept, times = lbm.lbm_batch_autotune(b, 20)
+        assert kept == 512 and sorted(times) == [128, 256, 512]
+        assert len(set(times.values())) == 1 and times[512] > 0
+    finally:
+        lbm.lbm_batch_destroy(b)
