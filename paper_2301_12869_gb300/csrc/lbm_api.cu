@@ -145,6 +145,7 @@ struct lbm_handle {
   // the populations f[cur] can be formed from m(1 - mcur), the state before the last step.
   lbm::WalkTiling walk{};
   bool walk_fits = false;  // its grid has a slot of the partial sums for every CTA
+  int step_band_w = 0, step_strip_h = 0;  // the population step's default tile on this lattice
   bool pop = true, mom = false;
   int mcur = 0;
   bool parts_ok = true;  // parts[pcur] are the partial sums of f[cur] (when not mom)
@@ -342,10 +343,15 @@ constexpr int kWalkSteps = 4;
 
 // The step on moments needs every relaxation time 1 and the default tile. FP64 lattices below
 // 2^16 nodes keep the population step: a walk's row takes 5 us of one warp's FP64 instructions
-// (4 x 200: 31.6 us a step against 13.6; 256 x 256: 48.6 against 52.1).
+// (4 x 200: 31.6 us a step against 13.6); beyond, the faster of the two is taken (walk_pays). With the
+// energy equation that is the walk: beside Heun's blocks the population step's do not all find an SM
+// at once (512 x 512: 192 us a step and 140, 32 x 2100 140 and 105).
 bool walk_usable(const lbm_handle* h) {
   return !h->graphs && h->walk_fits && lbm::unit_relaxation(h->phys) &&
-         (h->p.precision == LBM_FP32 || h->N >= (size_t(1) << 16));
+         (h->p.precision == LBM_FP32 ||
+          (h->N >= (size_t(1) << 16) &&
+           (h->p.thermal || lbm::walk_pays(h->p.precision, h->walk, h->nsm, h->step_band_w, h->step_strip_h,
+                                           h->p.gravity_form))));
 }
 bool walk_eligible(const lbm_handle* h) { return h->tiling.variant == 0 && walk_usable(h); }
 
@@ -682,6 +688,8 @@ int lbm_init(const lbm_params* p, const double* rho0, int rho0_where, void* stre
   if ((rc = lbm::prepare_step_kernels(h->dev, p->precision, h->err))) return fail(rc);
   if ((rc = plan_tiling(*p, h->nsm, &h->tiling, h->err))) return fail(rc);
   cudaError_t e = cudaSuccess;
+  h->step_band_w = h->tiling.band_w;
+  h->step_strip_h = h->tiling.strip_h;
   h->P = h->tiling.nbands * h->tiling.nstrips;
   h->Pcap = max_partials(*p, h->nsm, h->err);
   if (h->Pcap < 0) return fail(LBM_EINVAL);

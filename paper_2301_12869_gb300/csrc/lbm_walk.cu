@@ -566,6 +566,24 @@ bool plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, Wa
   return t->ctas <= max_ctas;
 }
 
+// FP32 walks win everywhere (24 B a node against 72). In FP64 both steps take the FP64 pipe's time, in
+// steps of whole rows, and which is less depends on how the rows fall out: 32 x 2100 walks in 49.2 us
+// a step and takes 30.9 on populations, 64 x 3000 81.8 and 58.2, 512 x 512 83.6 and 81.0, 60 x 1200
+// 34.1 and 38.7 (with <rho>), 1024 x 1024 227 and 255, 4 x 20000 84 and 190. Estimates, fitted to 75
+// lattices of 6e4 to 4e6 nodes (population step within 3 %, walk within 10 %): a row of the walk with w
+// warps on an SM takes max(5.8, 0.6 + 1.45 w) us, a population step's row 1.65 + 5 us a warp of 32
+// columns; <rho> costs that step 4 us, and the walk nothing (its own warp's). The walk has to win
+// by 5 %, since a block of steps also forms the moments and, when they are read, the populations: four
+// steps and a read of 100 x 3000 took 635 us, 432 on populations, where a step takes 101 and 103.
+bool walk_pays(int precision, const WalkTiling& t, int nsm, int step_band_w, int step_strip_h, int form) {
+  if (precision == 1) return true;
+  const int waves = (t.ctas + nsm - 1) / nsm;
+  const double walk = waves * ((t.strip_h + 6) / 3 * 3 * std::max(5.8, 0.6 + 1.45 * (t.threads / 32)) - 4.0);
+  const int w = (step_band_w + 31) / 32;
+  const double step = 9.3 + 1.4 * w + (1.65 + 5.0 * w) * step_strip_h + (form == 2 ? 4.0 : 0.0);
+  return walk < 0.95 * step;
+}
+
 namespace {
 template <typename T, int MODE, bool TH>
 cudaError_t launch_walk_m(const WalkTiling& t, const StepPhys& ph, const WalkIO& io, cudaStream_t s) {
