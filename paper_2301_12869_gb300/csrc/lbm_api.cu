@@ -586,7 +586,8 @@ int prepare_step_kernels(int dev, int precision, char* err) {
   }
   std::atomic<bool>& r = ready[dev][precision == LBM_FP32 ? 1 : 0];
   if (!r.load(std::memory_order_acquire)) {  // two threads may both set it: the same values
-    const cudaError_t e = step_prepare(precision);
+    cudaError_t e = step_prepare(precision);
+    if (e == cudaSuccess) e = walk_prepare(precision);
     if (e != cudaSuccess) {
       set_err(err, "kernel attributes: %s", cudaGetErrorString(e));
       return LBM_ECUDA;

@@ -109,6 +109,7 @@ bool plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, Wa
 // whether a step of that tiling is faster than the population step with the default tile, whose bands
 // are step_band_w columns wide and strips step_strip_h rows high
 bool walk_pays(int precision, const WalkTiling& t, int nsm, int step_band_w, int step_strip_h, int form);
+cudaError_t walk_prepare(int precision);  // sets the dynamic shared memory limit
 cudaError_t launch_walk(int precision, int mode, const WalkTiling& t, const StepPhys& ph, const WalkIO& io,
                         cudaStream_t stream);
 // M_t of the populations f*_t, and its partial sums (one per CTA of the tiling)

@@ -585,11 +585,19 @@ bool walk_pays(int precision, const WalkTiling& t, int nsm, int step_band_w, int
 }
 
 namespace {
+// FP64 thermal steps ask for more than half of an SM's shared memory, which they do not use, so that an
+// SM takes one of their blocks. The next step's blocks start beside the last ones of Heun's kernel, and
+// without that two of them (one has 3 to 8 warps) land on an SM that Heun has left while others get none:
+// 1024 x 1024 628 us a step in a block of steps for walk 240 and Heun 216 alone, 448 with it; 470 x 992
+// 317 and 222. Blocks of an isothermal step or an FP32 one come out the same either way.
+template <typename T, int MODE, bool TH>
+constexpr int kWalkShared = sizeof(T) == 8 && TH && MODE == WALK_STEP ? 120 * 1024 : 0;
+
 template <typename T, int MODE, bool TH>
 cudaError_t launch_walk_m(const WalkTiling& t, const StepPhys& ph, const WalkIO& io, cudaStream_t s) {
   const auto k = to_unit<typename LaneOf<T>::V>(ph);
-  return ph.form == 2 ? launch_dependent(walk_kernel<T, MODE, TH, true>, dim3(t.ctas), dim3(t.threads), 0, s, t, k, io)
-                      : launch_dependent(walk_kernel<T, MODE, TH, false>, dim3(t.ctas), dim3(t.threads), 0, s, t, k, io);
+  auto fn = ph.form == 2 ? walk_kernel<T, MODE, TH, true> : walk_kernel<T, MODE, TH, false>;
+  return launch_dependent(fn, dim3(t.ctas), dim3(t.threads), kWalkShared<T, MODE, TH>, s, t, k, io);
 }
 template <typename T>
 cudaError_t launch_walk_t(int mode, const WalkTiling& t, const StepPhys& ph, const WalkIO& io, cudaStream_t s) {
@@ -602,6 +610,15 @@ cudaError_t launch_walk_t(int mode, const WalkTiling& t, const StepPhys& ph, con
   return th ? launch_walk_m<T, WALK_MOMENTS, true>(t, ph, io, s) : launch_walk_m<T, WALK_MOMENTS, false>(t, ph, io, s);
 }
 }  // namespace
+
+cudaError_t walk_prepare(int precision) {
+  if (precision == 1) return cudaSuccess;
+  constexpr int bytes = kWalkShared<double, WALK_STEP, true>;
+  const cudaError_t e = cudaFuncSetAttribute(walk_kernel<double, WALK_STEP, true, false>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(walk_kernel<double, WALK_STEP, true, true>,
+                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
 
 cudaError_t launch_walk(int precision, int mode, const WalkTiling& t, const StepPhys& ph, const WalkIO& io,
                         cudaStream_t stream) {
