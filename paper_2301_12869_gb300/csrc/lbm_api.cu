@@ -362,10 +362,17 @@ bool walk_eligible(const lbm_handle* h) { return h->tiling.variant == 0 && walk_
 // against 12.9: a node a lane is 99 FP64 instructions of 61 clocks). A launch loads and stores the
 // populations, 8 to 11 us, so a call has to have some steps: FP32 64 x 256 in calls of 4 steps takes
 // 5.7 us a step and walks in 4.7, of 8 4.4 and 4.6; FP64 4 x 500 in calls of 4 steps 10.8.
+// A row takes a power of two of lanes, and the idle ones count: 100 x 160 FP32 (128 x 160) took 75 us
+// for 8 steps with <rho> between wet walls, 73 on populations, 50 walked; in FP64 24 x 80 (32 x 80) takes
+// 11.5 us a step as on populations, 20 x 100 13.1 against 11.3.
 constexpr int kColumnStepsF = 8, kColumnStepsD = 4;
 bool column_fits(const lbm_params& p) {
   const long long n = (long long)p.nx * p.ny;
   return !p.thermal && n <= (p.precision == LBM_FP32 ? 1 << 14 : 1 << 11);
+}
+bool column_pays(const lbm_params& p, const lbm::ColumnPlan& plan) {
+  const long long padded = ((p.precision == LBM_FP32 ? 4LL : 1LL) << plan.row_log2) * p.ny;
+  return padded <= (p.precision == LBM_FP32 ? 1 << 14 : 3 << 10);
 }
 bool column_usable(const lbm_handle* h) { return h->column.ok && lbm::unit_relaxation(h->phys); }
 
@@ -696,6 +703,7 @@ int lbm_init(const lbm_params* p, const double* rho0, int rho0_where, void* stre
   if (h->Pcap < 0) return fail(LBM_EINVAL);
   if (column_fits(*p)) {
     h->column = lbm::plan_columns(p->precision, p->nx, p->ny, p->ny, 8, p->precision == LBM_FP32 ? 0 : 64);
+    if (h->column.ok) h->column.ok = column_pays(*p, h->column);
     if (h->column.ok) h->column.ok = lbm::column_clusters(p->precision, h->column, false) > 0;
   }
   h->walk_fits = lbm::plan_walk(p->precision, p->nx, p->ny, p->wall == LBM_WALL_ZOU_HE, h->nsm, h->Pcap, &h->walk);

@@ -59,3 +59,23 @@ def test_mass_of_a_state_on_moments(form, zh):
         assert lbm.lbm_reduce(h, lbm.LBM_REDUCE_MASS)[0] == pytest.approx(float(np.sum(got)), rel=1e-13)
     finally:
         lbm.lbm_destroy(h)
+
+
+@pytest.mark.parametrize("nx, ny, precision, steps, chip", [
+    (100, 160, "fp32", 8, False), (20, 800, "fp32", 8, False), (64, 256, "fp32", 8, True), (100, 128, "fp32", 8, True),
+    (20, 100, "fp64", 4, False), (24, 80, "fp64", 4, True)])
+def test_padded_rows_count_for_the_steps_on_chip(nx, ny, precision, steps, chip):
+    """A row on chip takes a power of two of lanes. Lattices that fill less than their share are
+    stepped as in calls too short for the chip: the same bits as such calls."""
+    p, _, rho0, f = setup(nx, ny, precision, 2, True)
+    out = []
+    for block in (steps, steps // 2):
+        h = lbm.lbm_init(p, rho0)
+        try:
+            lbm.lbm_set_state(h, f)
+            for _ in range(0, steps, block):
+                lbm.lbm_step(h, block)
+            out.append(read(h, p))
+        finally:
+            lbm.lbm_destroy(h)
+    assert np.array_equal(*out) != chip
