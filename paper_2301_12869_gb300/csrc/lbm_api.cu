@@ -476,7 +476,6 @@ int settle(lbm_handle* h) {
 }
 
 int form_populations(lbm_handle* h) {
-  h->since_io = 0;
   if (int rc = settle(h)) return rc;
   if (h->graphs || h->pop) return LBM_OK;
   if (int rc = launch_populations(h, nullptr)) return rc;
@@ -916,6 +915,7 @@ int lbm_get_state(lbm_handle* h, double* f, int where, int64_t* steps_done) {
   if (!f || (where != LBM_HOST && where != LBM_DEVICE)) { set_err(h->err, "bad f or where"); return LBM_EINVAL; }
   if (steps_done) *steps_done = h->steps;
   if (int rc = form_populations(h)) return rc;
+  h->since_io = 0;
   if (where == LBM_DEVICE) {
     LBM_CUDA(h, lbm::launch_state_out(h->p.precision, h->f[h->cur], f, h->N, h->p.rho_ref, h->stream));
     return LBM_OK;

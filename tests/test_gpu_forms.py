@@ -79,3 +79,20 @@ def test_padded_rows_count_for_the_steps_on_chip(nx, ny, precision, steps, chip)
         finally:
             lbm.lbm_destroy(h)
     assert np.array_equal(*out) != chip
+
+
+@pytest.mark.parametrize("nx, ny, precision", [(256, 200, "fp32"), (64, 64, "fp32"), (260, 300, "fp64")])
+def test_single_steps_without_reads_walk(nx, ny, precision):
+    """From the fourth step on, steps in calls of one are steps on moments like a block's."""
+    p, _, rho0, f = setup(nx, ny, precision, 2, False)
+    out = []
+    for calls in ([1] * 10, [1, 1, 1, 7], [10]):
+        h = lbm.lbm_init(p, rho0)
+        try:
+            lbm.lbm_set_state(h, f)
+            for n in calls:
+                lbm.lbm_step(h, n)
+            out.append(read(h, p))
+        finally:
+            lbm.lbm_destroy(h)
+    assert np.array_equal(out[0], out[1]) and not np.array_equal(out[0], out[2])
