@@ -531,21 +531,23 @@ bool plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, Wa
   t->band_w = ((nx + t->nbands - 1) / t->nbands + W - 1) / W * W;
   t->nbands = (nx + t->band_w - 1) / t->band_w;
   const int most_warps = (fp32 ? kWalkThreadsF : kWalkThreadsD) / 32;
+  // warps a CTA takes: a share of an SM, or more where the partial sums' slots bound the grid (1024 x 30
+  // FP32 between wet walls has 60 for 180 warps in strips of 3 rows)
   auto set_rows = [&](int h) {
     t->strip_h = h;
     t->nstrips = (ny + h - 1) / h;
     const long warps = (long(t->nstrips) * t->nbands * t->seg + 31) / 32;
-    const int per_cta = int(std::min<long>(most_warps, (warps + nsm - 1) / nsm));
+    const long share = (warps + nsm - 1) / nsm, slots = std::max(max_ctas, 1);
+    const int per_cta = int(std::min<long>(most_warps, std::max(share, (warps + slots - 1) / slots)));
     t->threads = 32 * per_cta;
     t->ctas = int((warps + per_cta - 1) / per_cta);
-    return warps;
+    return t->ctas <= max_ctas;
   };
   double best = 0.0;
-  int best_h = 1;
+  int best_h = ny;
   for (int h = 1; h <= ny; h = h < 32 ? h + 1 : h + h / 16) {
-    const long per_sm = (set_rows(h) + nsm - 1) / nsm;
-    const double waves = double((per_sm + most_warps - 1) / most_warps);
-    const double w = double(std::min<long>(per_sm, most_warps));
+    if (!set_rows(h)) continue;
+    const double waves = double((t->ctas + nsm - 1) / nsm), w = double(t->threads / 32);
     const double row = fp32 ? 0.18 + 0.02 * w : std::max(5.0, 1.57 * w);
     const double time = waves * (1.4 + (h + 6) / 3 * 3 * row);
     if (best == 0.0 || time < best) {
@@ -553,17 +555,7 @@ bool plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, Wa
       best_h = h;
     }
   }
-  set_rows(best_h);
-  // the partial sums' slots bound the grid: taller strips, and where a strip is the whole height
-  // (wide lattices of a few rows: 4096 x 8 FP32 has 64 slots for 69 warps) more warps a CTA
-  while (t->ctas > max_ctas && t->strip_h < ny) set_rows(std::min(ny, t->strip_h + std::max(1, t->strip_h / 8)));
-  if (t->ctas > max_ctas && max_ctas > 0) {
-    const long warps = (long(t->nstrips) * t->nbands * t->seg + 31) / 32;
-    const int per_cta = int(std::min<long>(most_warps, (warps + max_ctas - 1) / max_ctas));
-    t->threads = 32 * per_cta;
-    t->ctas = int((warps + per_cta - 1) / per_cta);
-  }
-  return t->ctas <= max_ctas;
+  return set_rows(best_h);
 }
 
 // FP32 walks win everywhere (24 B a node against 72). In FP64 both steps take the FP64 pipe's time, in

@@ -59,3 +59,14 @@ def test_a_slot_for_every_cta(plan, precision, nx, ny):
 def test_too_few_slots_are_reported(plan, slots):
     ok, t = plan(FP32, 4096, 8, True, slots)  # 69 warps of at most 16 a CTA
     assert not ok and t.ctas > slots
+
+
+@pytest.mark.parametrize("precision, nx, ny, slots", [(FP32, 1024, 30, 60), (FP32, 424, 38, 38), (FP32, 308, 7, 7),
+                                                      (FP64, 1256, 13, 130)])
+def test_few_slots_take_more_warps_a_cta_before_taller_strips(plan, precision, nx, ny, slots):
+    """A step's time is its strip's rows (and six of halo and rounding); warps beside each other cost
+    little, so a grid that the slots bound keeps the strips it would have without them."""
+    ok, free = plan(precision, nx, ny, True, 1 << 20)
+    assert ok
+    ok, t = plan(precision, nx, ny, True, slots)
+    assert ok and t.ctas <= slots and t.strip_h <= free.strip_h + 2
