@@ -151,6 +151,7 @@ struct lbm_handle {
   bool parts_ok = true;  // parts[pcur] are the partial sums of f[cur] (when not mom)
   lbm::ColumnPlan column{};  // a small lattice is stepped on chip (ok: it fits)
   int since_io = 0;      // population steps since the populations were last set or read
+  bool pop_read = false; // they were what was read last (beside rho, u of the same state)
   // What a stream capture records runs at every replay, without the host's knowledge, so none of the
   // flags above may depend on it: from the first captured call on the populations f[cur] are the only
   // form, and parts[pcur] their sums after every call, as the calls in a graph find and leave them. A
@@ -335,10 +336,7 @@ int device_status(lbm_handle* h) {
 // Fewest steps from a populations state for which the moments are formed: the change of form
 // costs a pull (48 B a node) and, when the populations are read, a collision (48 B) on top of
 // 24 B a step against the population step's 72 B, so it pays from two steps on; up to four,
-// its two launches cost a small lattice what the steps save. The same holds for a state that has both
-// forms because its populations were read: fewer steps than that until the next read are population
-// steps (a step and a read in turn after a block, 1024 x 4096: FP64 2211 us walking and forming the
-// populations again, 1077 on populations; FP32 166 and 158; 256 x 768 FP32 30 and 31).
+// its two launches cost a small lattice what the steps save. (After a read of the populations: walks().)
 constexpr int kWalkSteps = 4;
 
 // The step on moments needs every relaxation time 1 and the default tile. FP64 lattices below
@@ -354,6 +352,20 @@ bool walk_usable(const lbm_handle* h) {
                                            h->p.gravity_form))));
 }
 bool walk_eligible(const lbm_handle* h) { return h->tiling.variant == 0 && walk_usable(h); }
+
+// Whether the next nsteps steps walk. Where the populations were read, the next read is expected after as
+// many steps again, and each route is charged with what it has to form for it. A step and a read in turn, us:
+// 1024 x 4096 FP64 1077 on populations and 2211 walking, FP32 158 and 166, 4 x 100000 FP32 460 and 39;
+// four steps and a read of 100 x 3000 FP64 432 and 635.
+bool walks(const lbm_handle* h, int64_t nsteps) {
+  if (!walk_eligible(h)) return false;
+  if (!h->pop) return true;
+  const int64_t n = nsteps + h->since_io;
+  if (!h->pop_read) return n >= kWalkSteps;
+  const lbm::StepCosts c = lbm::step_costs(h->p.precision, h->walk, h->nsm, h->step_band_w, h->step_strip_h,
+                                           h->p.gravity_form, h->p.thermal != 0);
+  return n * c.walk + c.populations + (h->mom ? 0.0 : c.pull) < n * c.step;
+}
 
 // Lattices small enough for one cluster are stepped on chip, a call's steps in a launch: FP32 up to
 // 2^14 nodes 128 wide (64 x 128 in calls of 64 steps: 2.6 us a step, 4.7 walked, 6.7 on populations;
@@ -535,6 +547,7 @@ int walk_launch(lbm_handle* h) {
 int walk_steps(lbm_handle* h, int64_t nsteps) {
   if (int rc = form_moments(h)) return rc;
   h->made = h->phys;
+  h->pop_read = false;
   for (int64_t t = 0; t < nsteps; ++t) {
     if (int rc = walk_launch(h)) return rc;
     h->pop = false;
@@ -547,6 +560,7 @@ int walk_steps(lbm_handle* h, int64_t nsteps) {
 
 int run_moments(lbm_handle* h, double* rho, double* ux, double* uy) {
   if (int rc = settle(h)) return rc;
+  if (h->since_io > 0) h->pop_read = false;
   const bool mom = h->mom && !h->graphs;
   if (mom && rho && !ux && !uy) {
     LBM_CUDA(h, lbm::launch_density(h->p.precision, h->phys, h->m(h->mcur), h->Tf, rho, h->N, h->status, h->stream));
@@ -788,8 +802,6 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
   if (nsteps < 0) { set_err(h->err, "nsteps must be >= 0"); return LBM_EINVAL; }
   if (nsteps == 0) return LBM_OK;
   if (int rc = settle(h)) return rc;
-  // not a single step between reads; a state read as populations goes on as populations then
-  const bool block = nsteps + h->since_io >= kWalkSteps;
   if (nsteps >= (h->p.precision == LBM_FP32 ? kColumnStepsF : kColumnStepsD) && h->tiling.variant == 0 &&
       column_usable(h)) {
     if (!h->graphs)
@@ -800,11 +812,11 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
     h->steps += nsteps;
     return h->graphs ? refresh_partials(h) : LBM_OK;  // a graph's next call may be any
   }
-  if (walk_eligible(h) && (block || !h->pop)) return walk_steps(h, nsteps);
+  if (walks(h, nsteps)) return walk_steps(h, nsteps);
   if (!h->graphs)
     if (int rc = leave_moments(h)) return rc;
   if (int rc = ensure_partials(h)) return rc;
-  h->since_io = int(std::min<int64_t>(h->since_io + nsteps, kWalkSteps));
+  h->since_io = int(std::min<int64_t>(h->since_io + nsteps, 1 << 20));
   lbm::StepIO io{};
   io.status = h->status;
   const lbm_params& p = h->p;
@@ -916,6 +928,7 @@ int lbm_get_state(lbm_handle* h, double* f, int where, int64_t* steps_done) {
   if (steps_done) *steps_done = h->steps;
   if (int rc = form_populations(h)) return rc;
   h->since_io = 0;
+  h->pop_read = true;
   if (where == LBM_DEVICE) {
     LBM_CUDA(h, lbm::launch_state_out(h->p.precision, h->f[h->cur], f, h->N, h->p.rho_ref, h->stream));
     return LBM_OK;
@@ -955,6 +968,7 @@ int lbm_set_state(lbm_handle* h, const double* f, int where, int64_t steps_done)
   h->npart = h->P;
   h->parts_ok = true;
   h->since_io = 0;
+  h->pop_read = false;
   h->have_prev = false;
   h->steps = steps_done;
   return LBM_OK;

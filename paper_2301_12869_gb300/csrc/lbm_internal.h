@@ -106,8 +106,15 @@ struct WalkIO {
 // the tiling of a lattice on a GPU of nsm SMs; at most max_ctas CTAs (partial sums), false where
 // that cannot be kept: such a tiling is not launched
 bool plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, WalkTiling* t);
-// whether a step of that tiling is faster than the population step with the default tile, whose bands
-// are step_band_w columns wide and strips step_strip_h rows high
+// estimated us of a step on moments and of the population step with the default tile, whose bands are
+// step_band_w columns wide and strips step_strip_h rows high; of forming the populations of a state on
+// moments, and the moments of one on populations
+struct StepCosts {
+  double walk, step, populations, pull;
+};
+StepCosts step_costs(int precision, const WalkTiling& t, int nsm, int step_band_w, int step_strip_h, int form,
+                     bool thermal);
+// whether steps without a read of the populations are to walk
 bool walk_pays(int precision, const WalkTiling& t, int nsm, int step_band_w, int step_strip_h, int form);
 cudaError_t walk_prepare(int precision);  // sets the dynamic shared memory limit
 cudaError_t launch_walk(int precision, int mode, const WalkTiling& t, const StepPhys& ph, const WalkIO& io,

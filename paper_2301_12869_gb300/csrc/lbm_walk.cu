@@ -558,22 +558,43 @@ bool plan_walk(int precision, int nx, int ny, bool zh, int nsm, int max_ctas, Wa
   return set_rows(best_h);
 }
 
+// Estimates in us, fitted to 75 lattices of 6e4 to 4e6 nodes in both gravity forms (FP64 population step
+// within 3 %, the walks within 10 %). A strip's rows, with six of halo and rounding, take a wave of the
+// walk 0.18 + 0.02 w us each with w warps on an SM, in FP64 max(5.8, 0.6 + 1.45 w); a row of the population
+// step 1.3 us (or the HBM's time for 72 B a node), in FP64 1.65 + 5 us a warp of 32 columns; FP64 thermal
+// ones of fewer than 3e5 nodes lose some 50 us beside Heun's blocks. Forming the populations is a walk with
+// nine planes to store, forming the moments a pass over memory.
+StepCosts step_costs(int precision, const WalkTiling& t, int nsm, int step_band_w, int step_strip_h, int form,
+                     bool thermal) {
+  const double nodes = double(t.nx) * t.ny, h = step_strip_h;
+  const int waves = (t.ctas + nsm - 1) / nsm, w = t.threads / 32, rows = (t.strip_h + 6) / 3 * 3;
+  StepCosts c;
+  if (precision == 1) {
+    c.walk = waves * (1.4 + rows * (0.18 + 0.02 * w)) + (form == 2 ? 2.0 : 0.0);
+    c.step = std::max(6.7 + 1.3 * h, 72.0 * nodes / 5.7e6);
+    c.populations = std::max(2.0 + 0.9 * c.walk, 48.0 * nodes / 6e6);
+    c.pull = 2.0 + 9e-6 * nodes;
+  } else {
+    const int n = (step_band_w + 31) / 32;
+    c.walk = waves * (rows * std::max(5.8, 0.6 + 1.45 * w) - 4.0);
+    const double r = step_strip_h == t.ny ? h - 0.8 : h;  // (the wall rows have no stencil)
+    c.step = 9.3 + 1.4 * n + (1.65 + 5.0 * n) * r + (form == 2 ? 4.0 : 0.0) + (thermal && nodes < 3e5 ? 50.0 : 0.0);
+    c.populations = 5.0 + 0.9 * c.walk;
+    c.pull = 8.0 + 3.6e-5 * nodes;
+  }
+  return c;
+}
+
 // FP32 walks win everywhere (24 B a node against 72). In FP64 both steps take the FP64 pipe's time, in
-// steps of whole rows, and which is less depends on how the rows fall out: 32 x 2100 walks in 49.2 us
-// a step and takes 30.9 on populations, 64 x 3000 81.8 and 58.2, 512 x 512 83.6 and 81.0, 60 x 1200
-// 34.1 and 38.7 (with <rho>), 1024 x 1024 227 and 255, 4 x 20000 84 and 190. Estimates, fitted to 75
-// lattices of 6e4 to 4e6 nodes (population step within 3 %, walk within 10 %): a row of the walk with w
-// warps on an SM takes max(5.8, 0.6 + 1.45 w) us, a population step's row 1.65 + 5 us a warp of 32
-// columns; <rho> costs that step 4 us, and the walk nothing (its own warp's). The walk has to win
-// by 5 %, since a block of steps also forms the moments and, when they are read, the populations: four
-// steps and a read of 100 x 3000 took 635 us, 432 on populations, where a step takes 101 and 103.
+// whole rows, and which is less depends on how the rows fall out: 32 x 2100 walks in 49.2 us a step and
+// takes 30.9 on populations, 64 x 3000 81.8 and 58.2, 512 x 512 83.6 and 81.0, 60 x 1200 34.1 and 38.7
+// (with <rho>), 1024 x 1024 227 and 255, 4 x 20000 84 and 190. Where they are alike the walk is taken:
+// the density of a state on moments costs nothing like a step (100 x 3000, a step and rho: 116 us, 190
+// on populations).
 bool walk_pays(int precision, const WalkTiling& t, int nsm, int step_band_w, int step_strip_h, int form) {
   if (precision == 1) return true;
-  const int waves = (t.ctas + nsm - 1) / nsm;
-  const double walk = waves * ((t.strip_h + 6) / 3 * 3 * std::max(5.8, 0.6 + 1.45 * (t.threads / 32)) - 4.0);
-  const int w = (step_band_w + 31) / 32;
-  const double step = 9.3 + 1.4 * w + (1.65 + 5.0 * w) * step_strip_h + (form == 2 ? 4.0 : 0.0);
-  return walk < 0.95 * step;
+  const StepCosts c = step_costs(precision, t, nsm, step_band_w, step_strip_h, form, false);
+  return c.walk < 1.05 * c.step;
 }
 
 namespace {

@@ -96,3 +96,30 @@ def test_single_steps_without_reads_walk(nx, ny, precision):
         finally:
             lbm.lbm_destroy(h)
     assert np.array_equal(out[0], out[1]) and not np.array_equal(out[0], out[2])
+
+
+@pytest.mark.parametrize("nx, ny, precision, steps, walk", [
+    (4, 3000, "fp32", 1, True), (512, 512, "fp32", 1, False), (256, 200, "fp32", 8, True), (12, 6000, "fp64", 1, False),
+    (12, 6000, "fp64", 4, True), (100, 3000, "fp64", 4, False), (1024, 256, "fp64", 1, False)])
+def test_steps_and_reads_in_turn_take_the_cheaper_route(nx, ny, precision, steps, walk):
+    """After a read of the populations: a population step's bits, or a walk's. us a turn on a GB300, on
+    populations and walking: 4 x 3000 FP32 37 and 23, 100 x 3000 FP64 with 4 steps 432 and 635."""
+    p, _, rho0, f = setup(nx, ny, precision, 1, False)
+    out = []
+    for route in ("turns", "walk", "populations"):
+        h = lbm.lbm_init(p, rho0)
+        try:
+            lbm.lbm_set_state(h, f)
+            lbm.lbm_step(h, 7)
+            if route == "populations":  # single steps from a state that was set
+                for _ in range(steps):
+                    lbm.lbm_set_state(h, read(h, p))
+                    lbm.lbm_step(h, 1)
+            else:
+                if route == "turns":
+                    read(h, p)
+                lbm.lbm_step(h, steps)
+            out.append(read(h, p))
+        finally:
+            lbm.lbm_destroy(h)
+    assert np.array_equal(out[0], out[1 if walk else 2]) and not np.array_equal(out[1], out[2])
