@@ -16,8 +16,8 @@
 // run parameters live in device memory so the graph is reused by every run.
 //
 // On chip against the general kernel (256 threads a column), us a step of the whole batch: 1024
-// columns of 64 and 128 rows FP32 21.0 -> 2.7, double-float 40.4 -> 18.8; 320 columns of 64 to
-// 1024 rows FP64 342 -> 104; 64 FP32 columns of 1000 rows 18.6 -> 2.7.
+// columns of 64 and 128 rows FP32 21.0 -> 2.8, double-float 40.4 -> 17.4; 320 columns of 64 to
+// 1024 rows FP64 342 -> 103; 64 FP32 columns of 1000 rows 18.6 -> 2.7.
 #include "lbm.h"
 #include "lbm_column.h"
 #include "lbm_internal.h"
@@ -543,7 +543,6 @@ __global__ void __launch_bounds__(256) batch_rest_kernel(const BatchArgs a) {
   }
 }
 
-// g_i = w_i (rho0 - rho_ref) for every column
 // rho_ref of every column: the mean of its density, summed in order (a thread a column: the value does
 // not depend on where rho0 lives). Of 1024 columns of 64 and 128 rows lbm_batch_init took 1215 us with
 // a device rho0 copied to the host and summed there, and takes 875
@@ -558,6 +557,7 @@ __global__ void __launch_bounds__(32) column_means_kernel(BatchCol* cols, int nc
   cols[c].rho_ref = s / double(n);
 }
 
+// g_i = w_i (rho0 - rho_ref) for every column
 template <typename T>
 __global__ void batch_init_kernel(const BatchCol* cols, int ncols, int nx, const double* rho0, T* f) {
   for (int c = blockIdx.x; c < ncols; c += gridDim.x) {

@@ -35,11 +35,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Waits for the phase with the given parity; gives up after `limit` clock cycles.
 // Programmatic dependent launch. A kernel launched with the programmatic stream
 // serialization attribute may start while the previous kernel in its stream is still
 // running; griddep_wait() returns once that kernel has completed and its writes are
-// visible, so nothing before it may touch global memory that kernel reads or writes.
+// visible, so nothing before it may write global memory, or read what that kernel writes.
+// A read ahead of it is safe only of what was complete before that kernel began to let others
+// start: what no kernel of the run writes, or what a kernel further back wrote, where the one
+// in between has itself waited (all its blocks, before griddep_launch_dependents()).
 // griddep_launch_dependents() lets the next kernel of the stream be scheduled (its blocks
 // take the resources of this kernel's blocks as they exit, and wait in turn).
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -48,8 +50,8 @@ __device__ __forceinline__ void griddep_launch_dependents() {
 }
 
 // Host side: launches fn as a programmatic dependent of the previous kernel in `stream`
-// (its launch and block set-up overlap that kernel's last blocks); fn must call
-// griddep_wait() before it touches global memory.
+// (its launch and block set-up overlap that kernel's last blocks); fn must call griddep_wait()
+// in every block, before what it reads or writes beyond the rule above.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_dependent(void (*fn)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                              Args&&... args) {
@@ -66,6 +68,7 @@ cudaError_t launch_dependent(void (*fn)(KArgs...), dim3 grid, dim3 block, size_t
   return cudaLaunchKernelEx(&cfg, fn, std::forward<Args>(args)...);
 }
 
+// Waits for the phase with the given parity; gives up after `limit` clock cycles.
 __device__ inline bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, long long limit = kWaitCycles) {
   if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();

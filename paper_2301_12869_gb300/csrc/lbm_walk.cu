@@ -10,9 +10,9 @@
 // Bound: 24 B a node and step against the population kernel's 72 B, and 87 operations a node
 // (packed in pairs for FP32) against 146. FP32 is bound by a row's dependency chain with 16
 // warps on an SM, FP64 by the FP64 pipe (an instruction per SM every 15.4 clocks). Measured
-// against the population step: 1024 x 4096 FP32 53.5 -> 22.5 us a step (4.5 TB/s of its own
-// 24 B), 772 x 1003 16.4 -> 5.9, 256 x 768 11.1 -> 5.9; 1024 x 4096 FP64
-// 1291 -> 821 us.
+// against the population step, steps alone: 1024 x 4096 FP32 with <rho> 53.1 -> 22.6 us a step (4.5
+// TB/s of its own 24 B), 772 x 1003 16.6 -> 6.2, 512 x 512 10.5 -> 4.3; 1024 x 4096 FP64 with <rho>
+// 1293 -> 819 us (971 on populations since they collide from three moments).
 //
 // Layout: a warp (or a segment of 8 or 16 lanes on narrow lattices) walks a strip of rows
 // upward. A lane holds two columns of a row, an FP32 pair or two FP64 values (two FP32 pairs a
@@ -182,8 +182,9 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? kWalkThreadsF : kWalkThreadsD
   // it). Warp 0 sums and announces it (bar.arrive) while the others form psi of their first rows,
   // and goes on to its own: nobody waits for warp 0's psi. Then only psi of the first two rows is
   // formed ahead of it, their collision is not needed (without <rho> there is nothing to wait for, and
-  // leaving those collisions out was slower: 772 x 1003 7.18 -> 7.29 us a step). 256 x 768 6.38 ->
-  // 6.25 us a step, 1024 x 4096 FP64 1018 -> 1007.
+  // leaving those collisions out was slower). Whole passes - a state set, a block of steps, the state and
+  // rho read - over their steps: 256 x 768 (200 steps) 6.38 -> 6.25 us, 1024 x 4096 FP64 (10) 1018 -> 1007;
+  // 772 x 1003 without <rho> (150) 7.18, without those collisions 7.29.
   const V zero = cst<V>(0.0);
   const L zero2 = splat_lane<V, N>(zero);
   V dmean = zero, dclose = zero;
