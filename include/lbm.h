@@ -128,14 +128,15 @@ int lbm_workspace_bytes(const lbm_params* p, uint64_t* bytes);
 int lbm_init(const lbm_params* p, const double* rho0, int rho0_where, void* stream, lbm_handle** out);
 
 /* Advance nsteps >= 0 time steps (asynchronous on the handle's stream). Each step is
- * one launch of a fused kernel - with every relaxation time 1 and the default tile one that
- * holds the state between calls as rho and j of the streamed populations, from which the
- * populations are formed when they are read; a call of several steps on a small lattice is one
+ * one launch of a fused kernel - with every relaxation time 1 and the default tile, where that is
+ * the faster one, one that holds the state between calls as rho and j of the streamed populations,
+ * from which the populations are formed when they are read; a call of several steps on a small lattice is one
  * launch that keeps the lattice on chip. Calls captured in a CUDA graph (an even number of steps a
  * graph) may be mixed with direct ones; from the first captured call on a handle's steps that are not
  * on chip are those on populations. A step: stream (and, with Zou-He walls, rebuild the wall nodes'
- * incoming populations), rho, psi, <rho>, F_int, F_g, u, MRT + Li forcing, store. Device-side faults (non-physical state, timeouts) are recorded in a
- * sticky status returned by the next synchronising call.
+ * incoming populations), rho, psi, <rho>, F_int, F_g, u, MRT + Li forcing,
+ * store. Device-side faults (non-physical state, timeouts) are recorded in a sticky status returned by
+ * the next synchronising call.
  * Thermal variant: psi uses R T(x) of the current temperature field T^n, and the step
  * also stores its rho^n and u^n; then one launch advances T^n by Heun's second-order
  * Runge-Kutta (dt = 1) on Eq. Energy_Equation with those rho^n, u^n held fixed,
